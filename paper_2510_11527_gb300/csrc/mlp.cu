@@ -9,9 +9,10 @@
 //     layers (mma.sync m16n8k16, FP32 accumulate, layer-1 accumulators reused as layer-2
 //     A fragments), FP32 output layer, softplus; one warp per 16 cells.
 //   features: training data (the same patch in FP32) and the plain indicator's label.
-//   train: per-sample FP32 forward (same bf16 rounding points as the tensor-core path)
-//     and backward, gradients accumulated per CTA in shared memory.
-//   adam: Adam update of the FP32 master weights and refresh of their bf16 copies.
+//   train: FP32 forward (same bf16 rounding points as the tensor-core path) and backward
+//     of tiles of 32 samples, gradients summed per CTA.
+//   adam: sum over the CTAs, Adam update of the FP32 master weights and refresh of their
+//     bf16 copies.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -61,38 +62,6 @@ __device__ __forceinline__ void normalise(const float v[NIN], float f[NIN]) {
   const float r = 1.0f / (sc + 1e-13f), m = v[4];
 #pragma unroll
   for (int k = 0; k < NIN; ++k) f[k] = (v[k] - m) * r;
-}
-
-// normalised patch of cell (i, j) in FP32: (v_k - ub_ij) / (max_k |v_k| + 1e-13)
-template <class PT>
-__device__ __forceinline__ void gather(const double* __restrict__ ub, const PT* __restrict__ V,
-                                       const PT* __restrict__ X, const PT* __restrict__ Y, int nx, int ny, int i,
-                                       int j, float f[NIN]) {
-  // patch offsets of the 13 cell averages (a along x, b along y)
-  constexpr int kPatchA[13] = {-1, 0, 1, -1, 0, 1, -1, 0, 1, -2, 2, 0, 0};
-  constexpr int kPatchB[13] = {-1, -1, -1, 0, 0, 0, 1, 1, 1, 0, 0, -2, 2};
-  float v[NIN];
-  // wrapped columns i-2..i+2 and row offsets j-2..j+2, formed once
-  int ci[5];
-  size_t rj[5];
-#pragma unroll
-  for (int d = 0; d < 5; ++d) {
-    ci[d] = wrapm(i + d - 2, nx);
-    rj[d] = (size_t)wrapm(j + d - 2, ny) * nx;
-  }
-#pragma unroll
-  for (int k = 0; k < 13; ++k) v[k] = af::to_stencil<float>(ub[rj[kPatchB[k] + 2] + ci[kPatchA[k] + 2]]);
-  const int im = ci[1], jm = wrapm(j - 1, ny);
-  const size_t c = (size_t)j * nx + i;
-  v[13] = to_f32(V[(size_t)jm * nx + im]);
-  v[14] = to_f32(V[(size_t)jm * nx + i]);
-  v[15] = to_f32(V[(size_t)j * nx + im]);
-  v[16] = to_f32(V[c]);
-  v[17] = to_f32(X[(size_t)j * nx + im]);
-  v[18] = to_f32(X[c]);
-  v[19] = to_f32(Y[(size_t)jm * nx + i]);
-  v[20] = to_f32(Y[c]);
-  normalise(v, f);
 }
 
 __device__ __forceinline__ float softplusf(float z) { return z > 20.0f ? z : log1pf(expf(z)); }
@@ -205,6 +174,54 @@ __device__ __forceinline__ void net_rows(const NetFrags& F, const __nv_bfloat16 
 #define AF_INDICATOR_MIN_CTAS 3
 #endif
 
+// The values of a 32 x 8 tile's patches in FP32: cell averages with a +-2 halo, points
+// with a -1 halo.
+struct PatchTile {
+  static constexpr int UX = 36, UY = 12, PX = 33, PY = 9;
+  float U[UY][UX], V[PY][PX], X[PY][PX], Y[PY][PX];
+};
+
+// stages the tile at (i0, j0) of a periodic mesh, by all 256 threads (no barrier); the
+// averages also as stored into dU [UY][UX] if given
+template <class PT>
+__device__ __forceinline__ void load_patch_tile(PatchTile& S, const double* __restrict__ ub,
+                                                const PT* __restrict__ V, const PT* __restrict__ X,
+                                                const PT* __restrict__ Y, int nx, int ny, int i0, int j0,
+                                                double* dU = nullptr) {
+  constexpr int UX = PatchTile::UX, UY = PatchTile::UY, PX = PatchTile::PX, PY = PatchTile::PY;
+  for (int k = threadIdx.x; k < UX * UY; k += 256) {
+    const int bx = k % UX, by = k / UX;
+    const double u = ub[(size_t)wrapm(j0 - 2 + by, ny) * nx + wrapm(i0 - 2 + bx, nx)];
+    S.U[by][bx] = af::to_stencil<float>(u);
+    if (dU) dU[k] = u;
+  }
+  for (int k = threadIdx.x; k < PX * PY; k += 256) {
+    const int bx = k % PX, by = k / PX;
+    const size_t g = (size_t)wrapm(j0 - 1 + by, ny) * nx + wrapm(i0 - 1 + bx, nx);
+    S.V[by][bx] = to_f32(V[g]);
+    S.X[by][bx] = to_f32(X[g]);
+    S.Y[by][bx] = to_f32(Y[g]);
+  }
+}
+
+// normalised patch of the tile's cell (tx, ty)
+__device__ __forceinline__ void patch_of(const PatchTile& S, int tx, int ty, float f[NIN]) {
+  constexpr int kPatchA[13] = {-1, 0, 1, -1, 0, 1, -1, 0, 1, -2, 2, 0, 0};
+  constexpr int kPatchB[13] = {-1, -1, -1, 0, 0, 0, 1, 1, 1, 0, 0, -2, 2};
+  float v[NIN];
+#pragma unroll
+  for (int k = 0; k < 13; ++k) v[k] = S.U[ty + 2 + kPatchB[k]][tx + 2 + kPatchA[k]];
+  v[13] = S.V[ty][tx];
+  v[14] = S.V[ty][tx + 1];
+  v[15] = S.V[ty + 1][tx];
+  v[16] = S.V[ty + 1][tx + 1];
+  v[17] = S.X[ty + 1][tx];
+  v[18] = S.X[ty + 1][tx + 1];
+  v[19] = S.Y[ty][tx + 1];
+  v[20] = S.Y[ty + 1][tx + 1];
+  normalise(v, f);
+}
+
 // One 32 x 8 tile (cells i0 .. i0 + 31, j0 .. j0 + 7) of a periodic mesh: the patches
 // are gathered into shared memory, each warp runs the network on its row of 32 cells
 // and writes s. Called by all 256 threads of the CTA, which it leaves synchronised.
@@ -213,41 +230,16 @@ __device__ __forceinline__ void indicator_tile(const NetFrags& F, const double* 
                                                const PT* __restrict__ V, const PT* __restrict__ X,
                                                const PT* __restrict__ Y, int nx, int ny, int i0, int j0,
                                                double* __restrict__ out) {
-  constexpr int UX = 36, UY = 12, PX = 33, PY = 9;
-  constexpr int kPatchA[13] = {-1, 0, 1, -1, 0, 1, -1, 0, 1, -2, 2, 0, 0};
-  constexpr int kPatchB[13] = {-1, -1, -1, 0, 0, 0, 1, 1, 1, 0, 0, -2, 2};
-  __shared__ float sU[UY][UX];
-  __shared__ float sV[PY][PX], sX[PY][PX], sY[PY][PX];
+  __shared__ PatchTile S;
   __shared__ __align__(16) __nv_bfloat16 sx[8][32][40];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   {
-    for (int k = tid; k < UX * UY; k += 256) {
-      const int bx = k % UX, by = k / UX;
-      sU[by][bx] = af::to_stencil<float>(ub[(size_t)wrapm(j0 - 2 + by, ny) * nx + wrapm(i0 - 2 + bx, nx)]);
-    }
-    for (int k = tid; k < PX * PY; k += 256) {
-      const int bx = k % PX, by = k / PX;
-      const size_t g = (size_t)wrapm(j0 - 1 + by, ny) * nx + wrapm(i0 - 1 + bx, nx);
-      sV[by][bx] = to_f32(V[g]);
-      sX[by][bx] = to_f32(X[g]);
-      sY[by][bx] = to_f32(Y[g]);
-    }
+    load_patch_tile<PT>(S, ub, V, X, Y, nx, ny, i0, j0);
     __syncthreads();
     {
       // cell (i0 + lane, j0 + warp)
-      const int tx = lane, ty = warp;
-      float v[NIN], f[NIN];
-#pragma unroll
-      for (int k = 0; k < 13; ++k) v[k] = sU[ty + 2 + kPatchB[k]][tx + 2 + kPatchA[k]];
-      v[13] = sV[ty][tx];
-      v[14] = sV[ty][tx + 1];
-      v[15] = sV[ty + 1][tx];
-      v[16] = sV[ty + 1][tx + 1];
-      v[17] = sX[ty + 1][tx];
-      v[18] = sX[ty + 1][tx + 1];
-      v[19] = sY[ty][tx + 1];
-      v[20] = sY[ty + 1][tx + 1];
-      normalise(v, f);
+      float f[NIN];
+      patch_of(S, lane, warp, f);
 #pragma unroll
       for (int k = 0; k < 32; k += 2)
         *reinterpret_cast<uint32_t*>(&sx[warp][lane][k]) =
@@ -340,29 +332,55 @@ __global__ void __launch_bounds__(256) infer_rows_kernel(const float* __restrict
   }
 }
 
-// training data: FP32 patch and the plain indicator max(s_1, s_2) (FP64) per cell
+// Training data: FP32 patch and the plain indicator max(s_1, s_2) (FP64) per cell, on
+// 32 x 8 tiles staged as the fused inference stages them. What bounds it is GB300's FP64
+// unit (the label's divisions): each s~ is formed once per location, 2.3 per cell instead
+// of the 6 of a cell by itself, and the patches, 21 floats per cell, leave through shared
+// memory so that a warp's 32 rows are one contiguous store.
 template <class PT>
-__global__ void features_kernel(const double* __restrict__ ub, const PT* __restrict__ V, const PT* __restrict__ X,
-                                const PT* __restrict__ Y, int nx, int ny, float* __restrict__ feat,
-                                float* __restrict__ label) {
-  const long long n = (long long)nx * ny;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(c % nx), j = (int)(c / nx);
-    float f[NIN];
-    gather<PT>(ub, V, X, Y, nx, ny, i, j, f);
-#pragma unroll
-    for (int k = 0; k < NIN; ++k) feat[c * NIN + k] = f[k];
+__global__ void __launch_bounds__(256) features_kernel(const double* __restrict__ ub, const PT* __restrict__ V,
+                                                       const PT* __restrict__ X, const PT* __restrict__ Y, int nx,
+                                                       int ny, float* __restrict__ feat, float* __restrict__ label) {
+  __shared__ PatchTile S;
+  __shared__ double dU[PatchTile::UY][PatchTile::UX];
+  __shared__ double st1[8][34], st2[10][32];   // s~_1 on columns -1 .. 32, s~_2 on rows -1 .. 8
+  __shared__ float rows[8][32 * NIN];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tiles_x = (nx + 31) / 32, tiles = tiles_x * ((ny + 7) / 8);
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const int i0 = (t % tiles_x) * 32, j0 = (t / tiles_x) * 8;
+    load_patch_tile<PT>(S, ub, V, X, Y, nx, ny, i0, j0, label ? &dU[0][0] : nullptr);
+    __syncthreads();
     if (label) {
-      auto U = [&](int a, int b) { return ub[(size_t)wrapm(j + b, ny) * nx + wrapm(i + a, nx)]; };
       auto st = [](double um, double uc, double up) {
         return fabs(um - 2.0 * uc + up) / (fabs(um) + 2.0 * fabs(uc) + fabs(up) + 1e-13);
       };
-      const double s1 = (st(U(-2, 0), U(-1, 0), U(0, 0)) + 4.0 * st(U(-1, 0), U(0, 0), U(1, 0)) +
-                         st(U(0, 0), U(1, 0), U(2, 0))) / 6.0;
-      const double s2 = (st(U(0, -2), U(0, -1), U(0, 0)) + 4.0 * st(U(0, -1), U(0, 0), U(0, 1)) +
-                         st(U(0, 0), U(0, 1), U(0, 2))) / 6.0;
-      label[c] = (float)fmax(s1, s2);
+      for (int k = tid; k < 8 * 34 + 10 * 32; k += 256) {
+        if (k < 8 * 34) {
+          const int x = k % 34, y = k / 34;
+          st1[y][x] = st(dU[y + 2][x], dU[y + 2][x + 1], dU[y + 2][x + 2]);
+        } else {
+          const int x = (k - 8 * 34) % 32, y = (k - 8 * 34) / 32;
+          st2[y][x] = st(dU[y][x + 2], dU[y + 1][x + 2], dU[y + 2][x + 2]);
+        }
+      }
     }
+    float f[NIN];
+    patch_of(S, lane, warp, f);
+#pragma unroll
+    for (int k = 0; k < NIN; ++k) rows[warp][lane * NIN + k] = f[k];
+    __syncthreads();
+    const int j = j0 + warp, w = min(32, nx - i0);
+    if (j < ny) {
+      const size_t c = (size_t)j * nx + i0;
+      for (int k = lane; k < w * NIN; k += 32) feat[c * NIN + k] = rows[warp][k];
+      if (label && lane < w) {
+        const double s1 = st1[warp][lane] + 4.0 * st1[warp][lane + 1] + st1[warp][lane + 2];
+        const double s2 = st2[warp][lane] + 4.0 * st2[warp + 1][lane] + st2[warp + 2][lane];
+        label[c + lane] = (float)(fmax(s1, s2) * (1.0 / 6.0));
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -375,95 +393,224 @@ __device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
   return z ^ (z >> 31);
 }
 
-// per-sample forward + backward in FP32 with the tensor-core path's rounding points
-// (bf16 inputs and weights of the two hidden layers); gradient of the batch-mean loss
-// accumulated into grad, loss into loss_acc. sample k of the batch is k itself when
-// seed == 0, else a splitmix64 draw over [0, nsamples).
-__global__ void __launch_bounds__(256) train_kernel(const float* __restrict__ feat, const float* __restrict__ label,
+// Forward + backward of a minibatch in FP32 with the tensor-core path's rounding points
+// (bf16 inputs and weights of the two hidden layers): the gradient of the batch-mean loss
+// summed over the samples of each CTA into its row of `partial` (TRAIN_ROW floats: the
+// parameters' gradient, then the loss), which adam_kernel / grad_kernel add up in a fixed
+// order, so a step is deterministic. Sample k of the batch is k itself when seed == 0,
+// else a splitmix64 draw over [0, nsamples).
+//
+// The work is a few thousand multiply-adds per sample: what bounds it is the length of one
+// thread's chain and how many SMs take part. One sample per thread with its 1793 shared
+// atomics took 0.5 ms per step of 4096 samples (16 CTAs); here a CTA takes tiles of 32
+// samples, lane = sample, and each of its 8 warps forms 4 of the 32 units of every layer
+// (weights as one broadcast 16-byte read per input), so 4096 samples are 128 CTAs and a
+// warp's chain is an eighth of the network's. The weight gradients are products of two
+// [unit][sample] arrays in shared memory, 4 + 3 entries per thread, kept in registers over
+// the CTA's tiles. Sums over a layer's inputs run in the order of the single-sample form.
+constexpr int TRAIN_TILE = 32;            // samples per tile (one per lane)
+constexpr int TRAIN_LD = TRAIN_TILE + 4;  // row stride: 16-byte aligned, 8 rows on distinct banks
+constexpr int TRAIN_MAX_CTAS = 152 * 2;   // rows of the partial sums
+constexpr int TRAIN_ROW = NPARAM + 7;     // 1800 floats per row: gradient, loss at NPARAM
+
+__global__ void __launch_bounds__(256, 2) train_kernel(const float* __restrict__ feat, const float* __restrict__ label,
                                                     long long nsamples, int batch, unsigned long long seed, int step,
-                                                    const float* __restrict__ params, float* __restrict__ grad,
-                                                    float* __restrict__ loss_acc) {
-  __shared__ float W1[NH * NIN], W2[NH * NH], b1[NH], b2[NH], w3[NH];
-  __shared__ float G[NPARAM];
-  __shared__ float b3s;
-  for (int k = threadIdx.x; k < NH * NIN; k += blockDim.x) W1[k] = bfr(params[OFF_W1 + k]);
-  for (int k = threadIdx.x; k < NH * NH; k += blockDim.x) W2[k] = bfr(params[OFF_W2 + k]);
-  for (int k = threadIdx.x; k < NH; k += blockDim.x) {
-    b1[k] = params[OFF_B1 + k];
-    b2[k] = params[OFF_B2 + k];
-    w3[k] = params[OFF_W3 + k];
+                                                    const float* __restrict__ params, float* __restrict__ partial) {
+  __shared__ __align__(16) float W1T[NIN][NH], W2T[NH][NH], W2[NH][NH];   // [input][unit], [input][unit], [unit][input]
+  __shared__ float b1[NH], b2[NH], w3[NH];
+  __shared__ __align__(16) float xT[NIN][TRAIN_LD], h1T[NH][TRAIN_LD], h2T[NH][TRAIN_LD];
+  __shared__ __align__(16) float d1T[NH][TRAIN_LD], d2T[NH][TRAIN_LD], d3[TRAIN_LD];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int k = tid; k < NH * NIN; k += 256) W1T[k % NIN][k / NIN] = bfr(params[OFF_W1 + k]);
+  for (int k = tid; k < NH * NH; k += 256) {
+    const float w = bfr(params[OFF_W2 + k]);
+    W2[k / NH][k % NH] = w;
+    W2T[k % NH][k / NH] = w;
   }
-  if (threadIdx.x == 0) b3s = params[OFF_B3];
-  for (int k = threadIdx.x; k < NPARAM; k += blockDim.x) G[k] = 0.f;
-  __syncthreads();
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  float lossv = 0.f;
-  if (k < batch) {
-    long long idx = seed == 0 ? k
-                              : (long long)(splitmix64(seed ^ ((unsigned long long)step << 32) ^ (unsigned long long)k) %
-                                            (unsigned long long)nsamples);
-    float x[NIN], z1[NH], h1[NH], z2[NH];
-    for (int q = 0; q < NIN; ++q) x[q] = bfr(feat[idx * NIN + q]);
-    for (int o = 0; o < NH; ++o) {
-      float a = 0.f;
-      for (int q = 0; q < NIN; ++q) a = fmaf(W1[o * NIN + q], x[q], a);
-      z1[o] = a + b1[o];
-      h1[o] = bfr(fmaxf(z1[o], 0.f));
+  if (tid < NH) {
+    b1[tid] = params[OFF_B1 + tid];
+    b2[tid] = params[OFF_B2 + tid];
+    w3[tid] = params[OFF_W3 + tid];
+  }
+  const float b3 = params[OFF_B3];
+  // this thread's gradient entries: W2 (unit go, inputs gq + 8 k), W1 (unit go, inputs
+  // gq + 8 k < 21) and one entry of b1, b2, w3 or b3
+  const int go = tid >> 3, gq = tid & 7;
+  float gw2[4] = {0.f, 0.f, 0.f, 0.f}, gw1[3] = {0.f, 0.f, 0.f}, gb = 0.f, lossv = 0.f;
+  const int tiles = (batch - 1) / TRAIN_TILE + 1;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const long long k = (long long)tile * TRAIN_TILE + lane;
+    const bool live = k < batch;
+    long long idx = 0;
+    if (live)
+      idx = seed == 0 ? k
+                      : (long long)(splitmix64(seed ^ ((unsigned long long)step << 32) ^ (unsigned long long)k) %
+                                    (unsigned long long)nsamples);
+    const float target = live ? label[idx] : 0.f;
+    __syncthreads();   // the previous tile's arrays have been read (and the weights written)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {   // rows 4 warp .. 4 warp + 3, one coalesced read each
+      const int sl = 4 * warp + r;
+      const long long row = __shfl_sync(0xffffffffu, idx, sl);
+      if (lane < NIN) xT[lane][sl] = k - lane + sl < batch ? bfr(feat[row * NIN + lane]) : 0.f;
     }
+    __syncthreads();
+    const int u0 = 4 * warp;   // this warp's units of each layer
+    float z1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < NIN; ++q) {
+      const float4 w = *reinterpret_cast<const float4*>(&W1T[q][u0]);
+      const float x = xT[q][lane];
+      z1[0] = fmaf(w.x, x, z1[0]);
+      z1[1] = fmaf(w.y, x, z1[1]);
+      z1[2] = fmaf(w.z, x, z1[2]);
+      z1[3] = fmaf(w.w, x, z1[3]);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      z1[e] += b1[u0 + e];
+      h1T[u0 + e][lane] = bfr(fmaxf(z1[e], 0.f));
+    }
+    __syncthreads();
+    float z2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < NH; ++q) {
+      const float4 w = *reinterpret_cast<const float4*>(&W2T[q][u0]);
+      const float h = h1T[q][lane];
+      z2[0] = fmaf(w.x, h, z2[0]);
+      z2[1] = fmaf(w.y, h, z2[1]);
+      z2[2] = fmaf(w.z, h, z2[2]);
+      z2[3] = fmaf(w.w, h, z2[3]);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      z2[e] += b2[u0 + e];
+      h2T[u0 + e][lane] = fmaxf(z2[e], 0.f);
+    }
+    __syncthreads();
+    // output layer and its gradient, formed by every warp for its lanes' samples
     float z3 = 0.f;
-    for (int o = 0; o < NH; ++o) {
-      float a = 0.f;
-      for (int q = 0; q < NH; ++q) a = fmaf(W2[o * NH + q], h1[q], a);
-      z2[o] = a + b2[o];
-      z3 = fmaf(w3[o], fmaxf(z2[o], 0.f), z3);
+#pragma unroll
+    for (int o = 0; o < NH; ++o) z3 = fmaf(w3[o], h2T[o][lane], z3);
+    z3 += b3;
+    const float r = softplusf(z3) - target;
+    const float dz3 = live ? 2.f / (float)batch * r / (1.f + expf(-z3)) : 0.f;
+    if (warp == 0) {
+      d3[lane] = dz3;
+      if (live) lossv += r * r / (float)batch;
     }
-    z3 += b3s;
-    const float out = softplusf(z3), r = out - label[idx];
-    lossv = r * r / (float)batch;
-    const float dz3 = 2.f / (float)batch * r / (1.f + expf(-z3));
-    atomicAdd(&G[OFF_B3], dz3);
-    float dh1[NH];
-    for (int q = 0; q < NH; ++q) dh1[q] = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) d2T[u0 + e][lane] = z2[e] > 0.f ? dz3 * w3[u0 + e] : 0.f;
+    __syncthreads();
+    float dh[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
     for (int o = 0; o < NH; ++o) {
-      atomicAdd(&G[OFF_W3 + o], dz3 * fmaxf(z2[o], 0.f));
-      if (z2[o] > 0.f) {
-        const float dz2 = dz3 * w3[o];
-        atomicAdd(&G[OFF_B2 + o], dz2);
-        for (int q = 0; q < NH; ++q) {
-          atomicAdd(&G[OFF_W2 + o * NH + q], dz2 * h1[q]);
-          dh1[q] = fmaf(dz2, W2[o * NH + q], dh1[q]);
+      const float4 w = *reinterpret_cast<const float4*>(&W2[o][u0]);
+      const float d = d2T[o][lane];
+      dh[0] = fmaf(d, w.x, dh[0]);
+      dh[1] = fmaf(d, w.y, dh[1]);
+      dh[2] = fmaf(d, w.z, dh[2]);
+      dh[3] = fmaf(d, w.w, dh[3]);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) d1T[u0 + e][lane] = z1[e] > 0.f ? dh[e] : 0.f;
+    __syncthreads();
+    // gradient entries of this tile
+#pragma unroll
+    for (int s = 0; s < TRAIN_TILE; s += 4) {
+      const float4 a2 = *reinterpret_cast<const float4*>(&d2T[go][s]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&d1T[go][s]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float4 h = *reinterpret_cast<const float4*>(&h1T[gq + 8 * e][s]);
+        gw2[e] = fmaf(a2.w, h.w, fmaf(a2.z, h.z, fmaf(a2.y, h.y, fmaf(a2.x, h.x, gw2[e]))));
+      }
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        if (gq + 8 * e < NIN) {
+          const float4 x = *reinterpret_cast<const float4*>(&xT[gq + 8 * e][s]);
+          gw1[e] = fmaf(a1.w, x.w, fmaf(a1.z, x.z, fmaf(a1.y, x.y, fmaf(a1.x, x.x, gw1[e]))));
         }
       }
     }
-    for (int q = 0; q < NH; ++q) {
-      if (z1[q] > 0.f) {
-        const float dz1 = dh1[q];
-        atomicAdd(&G[OFF_B1 + q], dz1);
-        for (int p = 0; p < NIN; ++p) atomicAdd(&G[OFF_W1 + q * NIN + p], dz1 * x[p]);
+    if (warp < 4) {
+      // b1, b2, w3 (unit = lane), b3 (lane 0 of warp 3)
+      const float* a = warp == 0 ? d1T[lane] : (warp == 1 ? d2T[lane] : (warp == 2 ? h2T[lane] : d3));
+      float acc = 0.f;
+      if (warp < 2 || (warp == 3 && lane == 0)) {
+        for (int s = 0; s < TRAIN_TILE; ++s) acc += a[s];
+      } else if (warp == 2) {
+        for (int s = 0; s < TRAIN_TILE; ++s) acc = fmaf(d3[s], a[s], acc);
       }
+      gb += acc;
     }
   }
-  for (int o = 16; o > 0; o >>= 1) lossv += __shfl_xor_sync(0xffffffffu, lossv, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss_acc, lossv);
-  __syncthreads();
-  for (int q = threadIdx.x; q < NPARAM; q += blockDim.x) atomicAdd(&grad[q], G[q]);
+  float* row = partial + (size_t)blockIdx.x * TRAIN_ROW;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) row[OFF_W2 + go * NH + gq + 8 * e] = gw2[e];
+#pragma unroll
+  for (int e = 0; e < 3; ++e)
+    if (gq + 8 * e < NIN) row[OFF_W1 + go * NIN + gq + 8 * e] = gw1[e];
+  if (warp == 0) {
+    row[OFF_B1 + lane] = gb;
+    for (int o = 16; o > 0; o >>= 1) lossv += __shfl_xor_sync(0xffffffffu, lossv, o);
+    if (lane == 0) row[NPARAM] = lossv;
+  } else if (warp == 1) {
+    row[OFF_B2 + lane] = gb;
+  } else if (warp == 2) {
+    row[OFF_W3 + lane] = gb;
+  } else if (warp == 3 && lane == 0) {
+    row[OFF_B3] = gb;
+  }
 }
 
-// Adam on the FP32 master weights; refreshes the bf16 copies and clears the gradient
-__global__ void adam_kernel(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                            float* __restrict__ grad, float lr, float c1, float c2, __nv_bfloat16* w1q,
-                            __nv_bfloat16* w2q) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= NPARAM) return;
-  const float g = grad[q];
+// sum over the CTAs' rows of column q = 32 blockIdx + lane (the gradient entries, then the
+// loss at NPARAM) in a fixed order: warp w takes rows w, w + 8, ..., then the warps in
+// order; valid in warp 0
+__device__ __forceinline__ float column_sum(const float* __restrict__ partial, int rows) {
+  __shared__ float sm[8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = blockIdx.x * 32 + lane;
+  float acc = 0.f;
+  if (q <= NPARAM) {
+#pragma unroll 4
+    for (int r = warp; r < rows; r += 8) acc += partial[(size_t)r * TRAIN_ROW + q];
+  }
+  sm[warp][lane] = acc;
+  __syncthreads();
+  float g = 0.f;
+  for (int w = 0; w < 8; ++w) g += sm[w][lane];
+  return g;
+}
+constexpr int COLUMN_CTAS = (NPARAM + 1 + 31) / 32;
+
+// Adam on the FP32 master weights with the gradient summed over the CTAs' rows; refreshes
+// the bf16 copies
+__global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ p, float* __restrict__ m,
+                                                   float* __restrict__ v, const float* __restrict__ partial, int rows,
+                                                   float lr, float c1, float c2, __nv_bfloat16* w1q,
+                                                   __nv_bfloat16* w2q, float* __restrict__ loss) {
+  const float g = column_sum(partial, rows);
+  const int q = blockIdx.x * 32 + (int)threadIdx.x;
+  if (threadIdx.x >= 32 || q > NPARAM) return;
+  if (q == NPARAM) {
+    *loss = g;
+    return;
+  }
   const float mq = 0.9f * m[q] + 0.1f * g, vq = 0.999f * v[q] + 0.001f * g * g;
   m[q] = mq;
   v[q] = vq;
   const float w = p[q] - lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
   p[q] = w;
-  grad[q] = 0.f;
   if (q < OFF_B1) w1q[(q / NIN) * 32 + q % NIN] = __float2bfloat16_rn(w);
   else if (q >= OFF_W2 && q < OFF_B2) w2q[q - OFF_W2] = __float2bfloat16_rn(w);
+}
+
+// the summed gradient (and the loss at NPARAM) alone
+__global__ void __launch_bounds__(256) grad_kernel(const float* __restrict__ partial, int rows,
+                                                   float* __restrict__ grad) {
+  const float g = column_sum(partial, rows);
+  const int q = blockIdx.x * 32 + (int)threadIdx.x;
+  if (threadIdx.x < 32 && q <= NPARAM) grad[q] = g;
 }
 
 __global__ void quantize_kernel(const float* __restrict__ p, __nv_bfloat16* w1q, __nv_bfloat16* w2q) {
@@ -482,8 +629,9 @@ struct af_mlp {
   float* params = nullptr;
   float* m = nullptr;
   float* v = nullptr;
-  float* grad = nullptr;
+  float* grad = nullptr;      // summed gradient, then the loss
   float* loss = nullptr;
+  float* partial = nullptr;   // TRAIN_MAX_CTAS rows of partial sums
   __nv_bfloat16* w1q = nullptr;
   __nv_bfloat16* w2q = nullptr;
   int t = 0;
@@ -518,6 +666,11 @@ cudaError_t mlp_indicator_batch_launch(const af_mlp* net, const BatchInst* inst,
 }
 }  // namespace af
 
+namespace {
+// CTAs (rows of partial sums) of a minibatch
+int train_rows(int batch) { return std::min((batch - 1) / TRAIN_TILE + 1, TRAIN_MAX_CTAS); }
+}  // namespace
+
 extern "C" {
 
 af_status af_mlp_create(af_mlp** out) {
@@ -527,7 +680,7 @@ af_status af_mlp_create(af_mlp** out) {
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) return AF_E_UNSUPPORTED;
   af_mlp* net = new (std::nothrow) af_mlp;
   if (!net) return AF_E_OOM;
-  const size_t bytes = 4 * 1024 * 5 * sizeof(float) + 2 * 32 * 32 * sizeof(__nv_bfloat16) + 256;
+  const size_t bytes = (10240 + TRAIN_MAX_CTAS * TRAIN_ROW) * sizeof(float) + 2 * 32 * 32 * sizeof(__nv_bfloat16) + 256;
   if (cudaMalloc(&net->block, bytes) != cudaSuccess) {
     cudaGetLastError();
     delete net;
@@ -540,7 +693,8 @@ af_status af_mlp_create(af_mlp** out) {
   net->v = f + 4096;
   net->grad = f + 6144;
   net->loss = f + 8192;
-  net->w1q = (__nv_bfloat16*)(f + 10240);
+  net->partial = f + 10240;
+  net->w1q = (__nv_bfloat16*)(net->partial + TRAIN_MAX_CTAS * TRAIN_ROW);
   net->w2q = net->w1q + 32 * 32;
   *out = net;
   return AF_OK;
@@ -559,7 +713,6 @@ af_status af_mlp_set_params(af_mlp* net, const float* host, int n) {
   if (cudaMemcpy(net->params, host, NPARAM * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) return AF_E_CUDA;
   cudaMemset(net->m, 0, NPARAM * sizeof(float));
   cudaMemset(net->v, 0, NPARAM * sizeof(float));
-  cudaMemset(net->grad, 0, NPARAM * sizeof(float));
   net->t = 0;
   quantize_kernel<<<4, 256>>>(net->params, net->w1q, net->w2q);
   return cudaDeviceSynchronize() == cudaSuccess ? AF_OK : AF_E_CUDA;
@@ -573,7 +726,8 @@ af_status af_mlp_get_params(const af_mlp* net, float* host) {
 
 af_status af_mlp_features(af_ctx* c, float* feat_dev, float* label_dev) {
   if (!c || !feat_dev || c->dim != 2 || c->bounds_pending) return AF_E_ARG;
-  const int grid = (int)std::min<size_t>((c->n + 255) / 256, 152 * 32);
+  const long long tiles = (long long)((c->nx + 31) / 32) * ((c->ny + 7) / 8);
+  const int grid = (int)std::min<long long>(tiles, 152 * 4);
   if (c->prec == AF_PREC_FP64)
     features_kernel<double><<<grid, 256, 0, c->stream>>>(c->ub[0], (const double*)c->pv[0], (const double*)c->px[0],
                                                          (const double*)c->py[0], c->nx, c->ny, feat_dev, label_dev);
@@ -601,16 +755,14 @@ af_status af_mlp_indicator(const af_mlp* net, af_ctx* c, double* s_dev) {
 af_status af_mlp_grad(af_mlp* net, const float* feat_dev, const float* label_dev, int nsamples, float* grad_host,
                       float* loss_host) {
   if (!net || !feat_dev || !label_dev || nsamples < 1) return AF_E_ARG;
-  cudaMemset(net->grad, 0, NPARAM * sizeof(float));
-  cudaMemset(net->loss, 0, sizeof(float));
-  train_kernel<<<(nsamples + 255) / 256, 256>>>(feat_dev, label_dev, nsamples, nsamples, 0ull, 0, net->params,
-                                               net->grad, net->loss);
+  const int rows = train_rows(nsamples);
+  train_kernel<<<rows, 256>>>(feat_dev, label_dev, nsamples, nsamples, 0ull, 0, net->params, net->partial);
+  grad_kernel<<<COLUMN_CTAS, 256>>>(net->partial, rows, net->grad);
   if (cudaGetLastError() != cudaSuccess) return AF_E_CUDA;
   if (grad_host && cudaMemcpy(grad_host, net->grad, NPARAM * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
     return AF_E_CUDA;
-  if (loss_host && cudaMemcpy(loss_host, net->loss, sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
+  if (loss_host && cudaMemcpy(loss_host, net->grad + NPARAM, sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
     return AF_E_CUDA;
-  cudaMemset(net->grad, 0, NPARAM * sizeof(float));
   return AF_OK;
 }
 
@@ -619,14 +771,13 @@ af_status af_mlp_train(af_mlp* net, const float* feat_dev, const float* label_de
   if (!net || !feat_dev || !label_dev || nsamples < 1 || batch < 1 || steps < 0 || !(lr > 0.f)) return AF_E_ARG;
   if (seed == 0 && batch > nsamples) return AF_E_ARG;   // seed 0: rows 0..batch-1 in order
   float last = 0.f;
+  const int rows = train_rows(batch);
   for (int s = 0; s < steps; ++s) {
-    cudaMemset(net->loss, 0, sizeof(float));
-    train_kernel<<<(batch + 255) / 256, 256>>>(feat_dev, label_dev, nsamples, batch, seed, s,
-                                               net->params, net->grad, net->loss);
+    train_kernel<<<rows, 256>>>(feat_dev, label_dev, nsamples, batch, seed, s, net->params, net->partial);
     net->t += 1;
     const float c1 = 1.f - powf(0.9f, (float)net->t), c2 = 1.f - powf(0.999f, (float)net->t);
-    adam_kernel<<<(NPARAM + 255) / 256, 256>>>(net->params, net->m, net->v, net->grad, lr, c1, c2, net->w1q,
-                                                net->w2q);
+    adam_kernel<<<COLUMN_CTAS, 256>>>(net->params, net->m, net->v, net->partial, rows, lr, c1, c2, net->w1q, net->w2q,
+                                      net->loss);
     if (cudaGetLastError() != cudaSuccess) return AF_E_CUDA;
     if (s == steps - 1 && loss_host) {
       if (cudaMemcpy(&last, net->loss, sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess) return AF_E_CUDA;

@@ -52,6 +52,23 @@ def test_features_and_labels_match_reference():
     np.testing.assert_allclose(lab.cpu().numpy(), ref_l, rtol=1e-6, atol=1e-7)
 
 
+@pytest.mark.parametrize("nx,ny,prec", [(1, 1, "fp64"), (5, 3, "fp32_mixed"), (33, 9, "fp64"), (70, 17, "fp32_mixed")])
+def test_features_on_ragged_tiles(nx, ny, prec):
+    """Meshes smaller than a tile's halo and with partly filled 32 x 8 tiles; FP32 points
+    are given as FP32 values, so both precisions hold the same inputs."""
+    from paper_2510_11527_gb300 import capi
+    spec = ai.Spec(dim=2, nx=nx, ny=ny, flux=("burgers", (0.5,)), umin=-1.0, umax=1.0)
+    st = [a.numpy() for a in ai.random_state_2d(spec, seed=nx, lo=-1, hi=1)]
+    st = [st[0]] + [a.astype(np.float32).astype(np.float64) for a in st[1:]]
+    with _ctx_with_state(spec, st, prec) as s:
+        feat = torch.full((spec.cells + 1, 21), 7.0, dtype=torch.float32, device="cuda")
+        lab = torch.full((spec.cells + 1,), 7.0, dtype=torch.float32, device="cuda")
+        capi.af_mlp_features(s.ctx, feat.data_ptr(), lab.data_ptr())
+    assert np.max(np.abs(feat[:-1].cpu().numpy() - mlp.features(*st))) <= 1e-6
+    np.testing.assert_allclose(lab[:-1].cpu().numpy(), mlp.plain_label(st[0]), rtol=1e-6, atol=1e-7)
+    assert bool((feat[-1] == 7.0).all()) and float(lab[-1]) == 7.0
+
+
 def _ref_forward(p, x32):
     return mlp.forward(mlp.unpack(p.astype(np.float64)), x32.astype(np.float64), quantize=True)[0]
 
@@ -163,6 +180,28 @@ def test_gradient_and_adam_step_match_reference():
         np.testing.assert_allclose(p1[big], pref[big], rtol=0, atol=1e-6)
     finally:
         capi.af_mlp_destroy(net)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4096, 32 * 304 + 5])
+def test_gradient_at_tile_edges(n):
+    """One sample, partly filled 32-sample tiles, and more tiles than CTAs: loss and
+    gradient against the reference, and the same bits twice."""
+    from paper_2510_11527_gb300 import capi
+    rng = np.random.default_rng(n)
+    x = rng.normal(0, 0.6, (n, 21)).astype(np.float32)
+    y = rng.uniform(0, 1, n).astype(np.float32)
+    net, p = _net(9)
+    try:
+        xd, yd = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
+        g, loss = capi.af_mlp_grad(net, xd.data_ptr(), yd.data_ptr(), n)
+        g2, loss2 = capi.af_mlp_grad(net, xd.data_ptr(), yd.data_ptr(), n)
+    finally:
+        capi.af_mlp_destroy(net)
+    lref, gref = mlp.loss_and_grad(mlp.unpack(p.astype(np.float64)), x.astype(np.float64), y.astype(np.float64), quantize=True)
+    gref = mlp.pack(gref)
+    assert loss == pytest.approx(lref, rel=1e-4)
+    assert np.max(np.abs(g - gref)) <= 1e-4 * np.max(np.abs(gref))
+    assert loss == loss2 and np.array_equal(g, g2)
 
 
 def _training_data(count=8, n=128, steps=4):
