@@ -194,16 +194,22 @@ int stage_plan(const af_ctx* c, int k, int* in, OutSpec out[2]) {
   }
 }
 
-// stage k of the configured scheme
+// arguments of stage k of the configured scheme (k in range)
 template <class PT>
-af_status stage_impl(af_ctx* c, int k) {
+StageArgs2D<PT> stage_args(af_ctx* c, int k) {
   int in = 0;
   OutSpec out[2];
   const int nout = stage_plan(c, k, &in, out);
-  if (nout == 0) FAIL(c, AF_E_ARG, "stage %d out of range", k);
   auto a = base_args<PT>(c, in);
   for (int o = 0; o < nout; ++o) set_out<PT>(c, a, o, out[o].oidx, out[o].cA, out[o].aidx, out[o].cF, out[o].tcoef, out[o].sg);
-  CK(c, launch<PT>(c, a));
+  return a;
+}
+
+// stage k of the configured scheme
+template <class PT>
+af_status stage_impl(af_ctx* c, int k) {
+  if (k < 0 || k >= af_num_stages(c)) FAIL(c, AF_E_ARG, "stage %d out of range", k);
+  CK(c, launch<PT>(c, stage_args<PT>(c, k)));
   return AF_OK;
 }
 
@@ -287,45 +293,53 @@ af_status stage_any(af_ctx* c, int k) {
   return c->prec == AF_PREC_FP64 ? stage_impl<double>(c, k) : stage_impl<float>(c, k);
 }
 
+// blocks of a rate reduction: one value per thread on small meshes, four CTAs per SM on
+// large ones
+int rate_blocks(size_t n) {
+  return (int)std::min<size_t>(152 * 4, (n + af::RED_THREADS - 1) / af::RED_THREADS);
+}
+
 template <int FLUX>
-cudaError_t launch_rate(af_ctx* c) {
-  const int blocks = 152 * 4;
+cudaError_t launch_rate(af_ctx* c, const af::DtFinal& fin) {
+  const int blocks = rate_blocks(FLUX == af::FLUX_ZERO || FLUX == af::FLUX_LINEAR ? 1 : c->pn);
   if constexpr (FLUX == af::FLUX_BL)
     af::dt_rate_kernel<FLUX><<<blocks, af::RED_THREADS, 0, c->stream>>>(c->m, c->dim, c->pnx, c->pny, c->inv_h1,
                                                                          c->inv_h2, c->kmax, c->ub[0], c->rate_bits,
-                                                                         c->grid.bc, c->grid.bc_left, c->grid.bc_right);
+                                                                         c->grid.bc, c->grid.bc_left, c->grid.bc_right,
+                                                                         fin);
   else
     af::dt_rate_maxu_kernel<FLUX><<<blocks, af::RED_THREADS, 0, c->stream>>>(
         c->m, c->dim, c->pnx, c->pny, c->inv_h1, c->inv_h2, c->kmax, c->ub[0], c->rate_bits, c->grid.bc,
-        c->grid.bc_left, c->grid.bc_right);
+        c->grid.bc_left, c->grid.bc_right, fin);
   return cudaGetLastError();
+}
+
+// how the CFL rate of a context becomes a step (see DtFinal)
+af::DtFinal dt_final(const af_ctx* c, double* dst, double* t_acc, double t_end, double* count) {
+  const double hmin = c->dim == 1 ? c->dx : (c->dim == 2 ? std::min(c->dx, c->dy) : std::min(c->dx, std::min(c->dy, c->dz)));
+  // no interior extrema of f_l' in 3D
+  return af::DtFinal{c->dim == 3 ? 0 : c->dim, c->inv_h1, c->inv_h2, c->cfl, c->cfl_diff, c->kmax,
+                     1.0 / (hmin * hmin), t_end, dst, t_acc, count};
 }
 
 // device CFL step -> *dst (no host round trip); t_acc: advance the device time
 af_status dt_device(af_ctx* c, double* dst, double* t_acc, double t_end = -1.0, double* count = nullptr) {
   cudaError_t e;
+  const af::DtFinal fin = dt_final(c, dst, t_acc, t_end, count);
   if (c->dim == 3) {
     const int n3[3] = {c->nx, c->ny, c->nz};
     const double ih3[3] = {c->inv_h1, c->inv_h2, c->inv_h3};
-    CK(c, af::launch_rate3d(c->flux.kind, c->m, n3, (const double*)c->k3[0][0], ih3, c->kmax, c->rate_bits, c->stream));
-    const double hmin = std::min(c->dx, std::min(c->dy, c->dz));
-    // no interior extrema of f_l' in 3D: the finalize step adds no extremum terms (dim 0)
-    af::dt_finalize_kernel<<<1, 1, 0, c->stream>>>(c->rate_bits, c->m, 0, c->inv_h1, c->inv_h2, c->cfl, c->cfl_diff,
-                                                   c->kmax, 1.0 / (hmin * hmin), dst, t_acc, t_end, count);
-    CK(c, cudaGetLastError());
+    CK(c, af::launch_rate3d(c->flux.kind, c->m, n3, (const double*)c->k3[0][0], ih3, c->kmax, c->rate_bits, fin,
+                            rate_blocks(c->n), c->stream));
     return AF_OK;
   }
   switch (c->flux.kind) {
-    case AF_FLUX_ZERO: e = launch_rate<af::FLUX_ZERO>(c); break;
-    case AF_FLUX_LINEAR: e = launch_rate<af::FLUX_LINEAR>(c); break;
-    case AF_FLUX_BURGERS: e = launch_rate<af::FLUX_BURGERS>(c); break;
-    default: e = launch_rate<af::FLUX_BL>(c); break;
+    case AF_FLUX_ZERO: e = launch_rate<af::FLUX_ZERO>(c, fin); break;
+    case AF_FLUX_LINEAR: e = launch_rate<af::FLUX_LINEAR>(c, fin); break;
+    case AF_FLUX_BURGERS: e = launch_rate<af::FLUX_BURGERS>(c, fin); break;
+    default: e = launch_rate<af::FLUX_BL>(c, fin); break;
   }
   CK(c, e);
-  const double hmin = c->dim == 1 ? c->dx : std::min(c->dx, c->dy);
-  af::dt_finalize_kernel<<<1, 1, 0, c->stream>>>(c->rate_bits, c->m, c->dim, c->inv_h1, c->inv_h2, c->cfl,
-                                                 c->cfl_diff, c->kmax, 1.0 / (hmin * hmin), dst, t_acc, t_end, count);
-  CK(c, cudaGetLastError());
   return AF_OK;
 }
 
@@ -351,6 +365,30 @@ af_status reduce_array(af_ctx* c, const S* x, size_t count, int op, double init,
   af::finalize_kernel<<<1, af::RED_THREADS, 0, c->stream>>>(c->partial, blocks, op, out_dev, accumulate);
   CK(c, cudaGetLastError());
   return AF_OK;
+}
+
+// short 1D meshes take whole steps in one launch
+bool marches(const af_ctx* c) { return c->dim == 1 && c->nx <= af::MARCH_MAX_CELLS; }
+
+// up to nsteps steps in one launch: of size dt > 0, or CFL steps clipped to t_end > 0
+template <class PT>
+af_status march_typed(af_ctx* c, int nsteps, double dt, double t_end, double* count) {
+  af::MarchArgs<PT> M;
+  M.nstages = af_num_stages(c);
+  M.nsteps = nsteps;
+  M.dt_fixed = dt;
+  M.fin = dt_final(c, c->dt_dev, c->t_dev, t_end, count);
+  for (int k = 0; k < M.nstages; ++k) M.st[k] = stage_args<PT>(c, k);
+  if constexpr (sizeof(PT) == 8) {
+    CK(c, af::launch_march1d_f64(c->flux.kind, c->m, M, c->stream));
+  } else {
+    CK(c, af::launch_march1d_f32(c->flux.kind, c->m, M, c->stream));
+  }
+  return AF_OK;
+}
+af_status march(af_ctx* c, int nsteps, double dt, double t_end = -1.0, double* count = nullptr) {
+  return c->prec == AF_PREC_FP64 ? march_typed<double>(c, nsteps, dt, t_end, count)
+                                 : march_typed<float>(c, nsteps, dt, t_end, count);
 }
 
 af_status set_dt(af_ctx* c, double dt, bool advance) {
@@ -467,7 +505,7 @@ af_status af_create(const af_grid* grid, const af_flux* flux, const af_diff* dif
   c->t_dev = (double*)p; p += al(8);
   c->red = (double*)p; p += al(8 * 8);
   c->partial = (double*)p; p += al(8 * af::RED_MAX_BLOCKS);
-  c->rate_bits = (unsigned long long*)p; p += al(16);
+  c->rate_bits = (unsigned long long*)p; p += al(24);
   c->stats = (DevStats*)p; p += al(sizeof(DevStats));
   c->s_ext = (double*)p; p += al(c->n * 8);
   for (int k = 0; d3 && k < 19; ++k) { c->scr3[k] = p; p += al(c->n * 8); }
@@ -760,11 +798,17 @@ af_status af_dt_device(af_ctx* c) {
 af_status af_step(af_ctx* c, double dt, double* dt_used) {
   if (!c || dt != dt) return AF_E_ARG;
   if (c->bounds_pending) FAIL(c, AF_E_STATE, "state not set");
-  af_status s = dt > 0.0 ? set_dt(c, dt, true) : dt_device(c, c->dt_dev, c->t_dev);
-  if (s != AF_OK) return s;
-  for (int k = 0; k < af_num_stages(c); ++k) {
-    s = stage_any(c, k);
+  af_status s;
+  if (marches(c)) {
+    s = march(c, 1, dt > 0.0 ? dt : 0.0);
     if (s != AF_OK) return s;
+  } else {
+    s = dt > 0.0 ? set_dt(c, dt, true) : dt_device(c, c->dt_dev, c->t_dev);
+    if (s != AF_OK) return s;
+    for (int k = 0; k < af_num_stages(c); ++k) {
+      s = stage_any(c, k);
+      if (s != AF_OK) return s;
+    }
   }
   if (dt_used) return read_scalar(c, c->dt_dev, dt_used);
   return AF_OK;
@@ -781,9 +825,14 @@ af_status af_run(af_ctx* c, double T, long long* nsteps) {
   // after T is reached have dt = 0, and a stage with dt = 0 writes nothing.
   double* count = c->red + 0;   // slot 0: step count of af_run
   CK(c, cudaMemsetAsync(count, 0, sizeof(double), c->stream));
-  const int chunk = 16;
+  // A mesh that marches takes a chunk in one launch, which ends when T is reached.
+  const int chunk = 16, march_chunk = 64;
   while (t < T * (1.0 - 1e-14)) {
-    for (int q = 0; q < chunk; ++q) {
+    if (marches(c)) {
+      s = march(c, march_chunk, 0.0, T, count);
+      if (s != AF_OK) return s;
+    }
+    for (int q = 0; q < chunk && !marches(c); ++q) {
       s = dt_device(c, c->dt_dev, c->t_dev, T, count);
       if (s != AF_OK) return s;
       for (int k = 0; k < af_num_stages(c); ++k) {

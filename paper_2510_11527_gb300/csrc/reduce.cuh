@@ -18,7 +18,7 @@ constexpr int RED_MAX_BLOCKS = 1024;   // partial-result slots per reduction
 // together with |f_l'(c)| / h + kappa_max / h^2 for each interior extremum c of f_l'
 // that lies strictly inside some face interval. The kernel reduces the first term into
 // rate_bits[0] (non-negative doubles order like their bit patterns) and flags the
-// extrema met (bit 8 l + k) in rate_bits[1]; dt_finalize_kernel adds their terms.
+// extrema met (bit 8 l + k) in rate_bits[1]; dt_finish adds their terms.
 // A bounded 1D interval (bc != AF_BC_PERIODIC) has no wrap-around face; its two end
 // faces join the end cells to their ghosts: the Dirichlet values gl / gr are then face
 // end points too, while an outflow ghost repeats the end cell (nothing new). A 2D
@@ -35,6 +35,61 @@ __device__ __forceinline__ unsigned crit_flags(const DevModel& m, int dir, doubl
   return f;
 }
 
+// rate over the flagged extrema (see dt_rate_kernel)
+__device__ __forceinline__ double crit_rate(const DevModel& m, int dim, double inv_h1, double inv_h2, double kmax,
+                                            unsigned long long flags, double rate) {
+  const double kd1 = kmax * inv_h1 * inv_h1, kd2 = kmax * inv_h2 * inv_h2;
+  for (int d = 0; d < dim; ++d)
+    for (int k = 0; k < m.ncrit[d]; ++k)
+      if ((flags >> (8 * d + k)) & 1ull)
+        rate = tmax(rate, d == 0 ? m.critv[0][k] * inv_h1 + kd1 : m.critv[1][k] * inv_h2 + kd2);
+  return rate;
+}
+
+// How a CFL rate becomes the step: where the step goes (dt_out), the simulated time it
+// advances (t_acc, optional), the end time it is clipped to (t_end > 0) and the count of
+// positive steps; crit_dim directions of interior extrema (0 in 3D: there are none).
+struct DtFinal {
+  int crit_dim;
+  double inv_h1, inv_h2, cfl, cfl_diff, kmax, inv_hmin2, t_end;
+  double* dt_out;
+  double* t_acc;
+  double* count;
+};
+
+// dt = 1 / max(rate / C, kappa_max / (h_min^2 Cd)); with t_end > 0 clipped to the time
+// left after t (0 once less than t_end * 1e-14 is left)
+__device__ __forceinline__ double cfl_step(const DevModel& m, const DtFinal& f, unsigned long long rate_bits,
+                                           unsigned long long flags, double t) {
+  const double rate =
+      crit_rate(m, f.crit_dim, f.inv_h1, f.inv_h2, f.kmax, flags, __longlong_as_double((long long)rate_bits));
+  double r = rate / f.cfl;
+  if (f.cfl_diff > 0.0 && f.kmax > 0.0) r = fmax(r, f.kmax * f.inv_hmin2 / f.cfl_diff);
+  double dt = r > 0.0 ? 1.0 / r : 0.0;
+  if (f.t_acc && f.t_end > 0.0) {
+    const double left = f.t_end - t;
+    dt = left > f.t_end * 1e-14 ? fmin(dt, left) : 0.0;
+  }
+  return dt;
+}
+
+// The end of a rate kernel, by thread 0 of each block after its atomics on acc[0] (rate
+// bits) and acc[1] (extremum flags): the block that arrives last (ticket acc[2]) forms
+// the step, advances the time and resets the accumulators for the next reduction. One
+// launch instead of two: the single-thread launch that did this by itself cost 3 us and a
+// gap of its own per step.
+__device__ __forceinline__ void dt_finish(unsigned long long* acc, const DevModel& m, const DtFinal& f) {
+  __threadfence();
+  if (atomicAdd(acc + 2, 1ull) != (unsigned long long)gridDim.x - 1ull) return;
+  __threadfence();
+  const unsigned long long bits = __ldcg(acc), flags = __ldcg(acc + 1);
+  const double dt = cfl_step(m, f, bits, flags, f.t_acc ? *f.t_acc : 0.0);
+  if (f.t_acc && f.t_end > 0.0 && dt > 0.0) *f.count += 1.0;
+  *f.dt_out = dt;
+  if (f.t_acc) *f.t_acc += dt;
+  acc[0] = acc[1] = acc[2] = 0ull;
+}
+
 // The same rate for a flux whose |f_l'| is a nondecreasing function of |u| (Burgers) or a
 // constant (linear, zero): rounding is monotone, so the largest rate is the rate at the
 // largest |u|. A maximum of the magnitude bits (integer units only) per block, the rate
@@ -44,7 +99,7 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_maxu_kernel(const DevMode
                                                                     double inv_h1, double inv_h2, double kmax,
                                                                     const double* __restrict__ ub,
                                                                     unsigned long long* rate_bits, int bc, double gl,
-                                                                    double gr) {
+                                                                    double gr, const DtFinal fin) {
   const size_t n = (size_t)nx * ny;
   const double kd1 = kmax * inv_h1 * inv_h1, kd2 = kmax * inv_h2 * inv_h2;
   const bool rect = dim == 2 && bc != AF_BC_PERIODIC;
@@ -79,6 +134,7 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_maxu_kernel(const DevMode
     double b = a1 * inv_h1 + kd1;
     if (dim == 2) b = tmax(b, a2 * inv_h2 + kd2);
     atomicMax(rate_bits, (unsigned long long)__double_as_longlong(b));
+    dt_finish(rate_bits, m, fin);
   }
 }
 
@@ -87,7 +143,7 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
                                                                double inv_h1, double inv_h2, double kmax,
                                                                const double* __restrict__ ub,
                                                                unsigned long long* rate_bits, int bc, double gl,
-                                                               double gr) {
+                                                               double gr, const DtFinal fin) {
   const size_t n = (size_t)nx * ny;
   double best = 0.0;
   unsigned flags = 0u;
@@ -183,41 +239,8 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
     }
     atomicMax(rate_bits, (unsigned long long)__double_as_longlong(b));
     if (f) atomicOr(rate_bits + 1, (unsigned long long)f);
+    dt_finish(rate_bits, m, fin);
   }
-}
-
-// rate over the flagged extrema (see dt_rate_kernel)
-__device__ __forceinline__ double crit_rate(const DevModel& m, int dim, double inv_h1, double inv_h2, double kmax,
-                                            unsigned long long flags, double rate) {
-  const double kd1 = kmax * inv_h1 * inv_h1, kd2 = kmax * inv_h2 * inv_h2;
-  for (int d = 0; d < dim; ++d)
-    for (int k = 0; k < m.ncrit[d]; ++k)
-      if ((flags >> (8 * d + k)) & 1ull)
-        rate = tmax(rate, d == 0 ? m.critv[0][k] * inv_h1 + kd1 : m.critv[1][k] * inv_h2 + kd2);
-  return rate;
-}
-
-// dt = 1 / max(rate / C, kappa_max / (h_min^2 Cd)). Resets the accumulators for the
-// next step. When t_acc is given the step is also added to the simulated time; with
-// t_end > 0 the step is first clipped to the time left before t_end (0 once less than
-// t_end * 1e-14 is left) and each positive step is counted in *count.
-static __global__ void dt_finalize_kernel(unsigned long long* rate_bits, const DevModel m, int dim, double inv_h1,
-                                          double inv_h2, double cfl, double cfl_diff, double kmax, double inv_hmin2,
-                                          double* dt_out, double* t_acc, double t_end, double* count) {
-  const double rate =
-      crit_rate(m, dim, inv_h1, inv_h2, kmax, rate_bits[1], __longlong_as_double((long long)rate_bits[0]));
-  double r = rate / cfl;
-  if (cfl_diff > 0.0 && kmax > 0.0) r = fmax(r, kmax * inv_hmin2 / cfl_diff);
-  double dt = r > 0.0 ? 1.0 / r : 0.0;
-  if (t_acc && t_end > 0.0) {
-    const double left = t_end - *t_acc;
-    dt = left > t_end * 1e-14 ? fmin(dt, left) : 0.0;
-    if (dt > 0.0) *count += 1.0;
-  }
-  *dt_out = dt;
-  if (t_acc) *t_acc += dt;
-  rate_bits[0] = 0ull;
-  rate_bits[1] = 0ull;
 }
 
 // *dt = v and, when t_acc is given, *t_acc += v

@@ -14,17 +14,35 @@
 // 4/dx^2 sum_{m,n} b_mn kappa(z_m) z_n on its line, and the limiter blends the total
 // face flux with F^L - (a(ub_{i+1}) - a(ub_i))/dx by Theta with factor 2.
 // A bounded interval (Dirichlet / outflow ends) reads ghost cells and points from the
-// boundary rule, updates the extra left end point u_{-1/2} in CTA 0, and holds
+// boundary rule, updates the extra left end point u_{-1/2} in its first tile, and holds
 // Dirichlet end points at the boundary values.
 #pragma once
-#include "stage2d.cuh"
+#include <cooperative_groups.h>
+
+#include "launch.h"
 
 namespace af {
 
-template <int FLUX, class T>
+// A tile of TX cells with a +-3 cell halo, worked on by NT threads. Two shapes: 256 cells
+// by 256 threads for long meshes, and 26 cells by one warp (halo included, one box
+// position per lane) for meshes that would otherwise leave most SMs idle: GB300's FP64
+// unit passes 2 lanes per clock and SM, so a short mesh is bound by the FP64 rate of the
+// few SMs it runs on (200 cells in one 256-cell tile: 17 us per stage, bound by one SM's
+// FP64 unit; 8 one-warp tiles on 8 SMs: see march1d_kernel).
+template <int TX_, int NT_>
 struct Tile1D {
-  static constexpr int TX = 256, NT = TX, H = 3, BX = TX + 2 * H;
+  static constexpr int TX = TX_, NT = NT_, H = 3, BX = TX + 2 * H;
+  static_assert(NT == TX || NT >= BX, "one thread per cell, or per box position");
 };
+using Tile1DLong = Tile1D<256, 256>;
+using Tile1DWarp = Tile1D<WARP_TILE_1D, 32>;
+
+// barrier among the threads of one tile
+template <int NT>
+__device__ __forceinline__ void tile_sync() {
+  if constexpr (NT == 32) __syncwarp();
+  else __syncthreads();
+}
 
 // Cell average ub_i and point value u_{j+1/2} at any index: stored values inside, the
 // boundary rule outside (periodic image; Dirichlet value; even reflection about the
@@ -76,33 +94,39 @@ struct Scal1D {
   int comb[2];
 };
 
-template <int FLUX, class T, class PT>
-__global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const StageArgs2D<PT> A) {
-  using L = Tile1D<FLUX, T>;
+// shared memory of one tile
+template <class T, int BX>
+struct Shared1D {
+  T U[BX], P[BX], C[BX];
+  // aP / aC hold kappa instead of a without double conservation (no DC potential)
+  T fP[BX], aP[BX], fC[BX], aC[BX], dP[BX], dC[BX], fU[BX], aU[BX];
+  T FH[BX], AH[BX], FL[BX], ULp[BX], ULm[BX], Flim[BX], Alim[BX];
+  T S[BX], TC[BX], TD[BX];
+  Scal1D<T> sc;
+};
+
+// One tile of cells i0 .. i0 + TX - 1 (tid: the thread's index in the tile): one or two
+// limited forward-Euler evaluations with step tcoef * dtv, their combination and store.
+template <int FLUX, class T, class PT, class L>
+__device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2D<PT>& A, double dtv, int i0, int tid,
+                                             Shared1D<T, L::BX>& sm) {
   constexpr int TX = L::TX, NT = L::NT, H = L::H, BX = L::BX;
   // flux direction of the model functions: the 1D Buckley-Leverett flux is the gravity
   // form f1 (1 - g (1-u)^2), which the model keeps as direction 1 (Example 6.6)
   constexpr int XD = FLUX == FLUX_BL ? 1 : 0;
-  __shared__ T sU[BX], sP[BX], sC[BX];
-  // aP / aC hold kappa instead of a without double conservation (no DC potential)
-  __shared__ T fP[BX], aP[BX], fC[BX], aC[BX], dP[BX], dC[BX], fU[BX], aU[BX];
-  __shared__ T sFH[BX], sAH[BX], sFL[BX], sULp[BX], sULm[BX], sFlim[BX], sAlim[BX];
-  __shared__ T sS[BX], sTC[BX], sTD[BX];
-
-  const double dtv = *A.dt;
-  if (is_zero_bits(dtv)) return;   // uniform over the grid
+  T *sU = sm.U, *sP = sm.P, *sC = sm.C, *fP = sm.fP, *aP = sm.aP, *fC = sm.fC, *aC = sm.aC, *dP = sm.dP, *dC = sm.dC,
+    *fU = sm.fU, *aU = sm.aU, *sFH = sm.FH, *sAH = sm.AH, *sFL = sm.FL, *sULp = sm.ULp, *sULm = sm.ULm,
+    *sFlim = sm.Flim, *sAlim = sm.Alim, *sS = sm.S, *sTC = sm.TC, *sTD = sm.TD;
+  Scal1D<T>& sc = sm.sc;
   const int nx = A.nx;
-  const int i0 = blockIdx.x * TX;
-  const int tid = threadIdx.x;
-  __shared__ Scal1D<T> sc;
   // formed at once by the lanes of warp o (output o) and the upper lanes of warp 0 (the
   // mesh's values): GB300's FP64 unit takes as long for a warp instruction with one
   // active lane as with 32. Lane l evaluates fl(fl(fl(x y1) y2) y3) with the factors of
   // its value's formula (a factor 1 is exact, so each value is rounded as its formula
   // is; the divided line scales come from the host); only the stores differ between
   // lanes.
-  if ((tid >> 5) < A.nout) {
-    const int o = tid >> 5, l = tid & 31;
+  for (int o = tid >> 5; o < A.nout; o += NT / 32) {
+    const int l = tid & 31;
     const double ih = A.inv_h1, tau = A.tcoef[o] * dtv;
     double x = tau, y1 = 1.0, y2 = 1.0, y3 = 1.0;
     if (l < 16) {
@@ -152,7 +176,7 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
       default: break;
     }
   }
-  __syncthreads();
+  tile_sync<NT>();
   const T umin = sc.umin, umax = sc.umax;
   const bool blend = A.blend != 0;
   const bool ext = A.blend == 2;
@@ -165,7 +189,7 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
     sU[k] = to_stencil_nb<T>(cell1d(A, i0 - H + k, H), m.umid);
     sP[k] = T(point1d(A, i0 - H + k, H));
   }
-  __syncthreads();
+  tile_sync<NT>();
   for (int b = tid; b < BX; b += NT) {
     const T u = sU[b];
     fU[b] = flux<FLUX, T>(m, XD, u);
@@ -186,14 +210,16 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
       sTC[b] = tabs(um - T(2) * u + up) / (tabs(um) + T(2) * tabs(u) + tabs(up) + T(1e-13));
     }
   }
-  __syncthreads();
+  tile_sync<NT>();
   const T ih = sc.ih, i6h = sc.i6h, i3h2 = sc.i3h2;
-  // points updated by this thread: its own u_{i+1/2} and, in CTA 0 of a bounded
+  // points updated by this thread: its own u_{i+1/2} and, in the first tile of a bounded
   // interval, thread 0 also the left end point u_{-1/2} (held at the boundary value
   // when the end is Dirichlet)
-  const bool extra = bounded && blockIdx.x == 0 && tid == 0;
-  const int nq = extra ? 2 : 1;
-  const int bq[2] = {H + tid, H - 1};
+  // (a one-warp tile gives it to a lane without a cell of its own instead)
+  constexpr bool SPARE = NT > TX;
+  const bool extra = bounded && i0 == 0 && tid == (SPARE ? TX : 0);
+  const int nq = SPARE ? (tid < TX || extra ? 1 : 0) : (extra ? 2 : 1);
+  const int bq[2] = {SPARE && tid >= TX ? H - 1 : H + tid, H - 1};
   // high-order point residual
   T rH[2] = {T(0), T(0)};
   for (int q = 0; q < nq; ++q) {
@@ -237,7 +263,7 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
       sS[b] = ext ? T(A.s_ext[wrapi(i0 - H + b, nx)]) : (sTC[b - 1] + T(4) * sTC[b] + sTC[b + 1]) * T(1.0 / 6.0);
     }
   }
-  __syncthreads();
+  tile_sync<NT>();
   T rP[2] = {rH[0], rH[1]};
   if (blend) {
     const T g = sc.g;
@@ -245,7 +271,7 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
       sTD[b] = exp(-g * sS[b]);
       if (b < H + TX) sTC[b] = exp(-g * (T(0.5) * (sS[b] + sS[b + 1])));
     }
-    __syncthreads();
+    tile_sync<NT>();
     for (int b = H - 1 + tid; b <= H + TX; b += NT) {
       if (b < H + TX) sFH[b] = sTC[b] * sFH[b] + (T(1) - sTC[b]) * sFL[b];
       sAH[b] = sTD[b] * sAH[b] + (T(1) - sTD[b]) * aU[b];
@@ -258,10 +284,10 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
       const T RL = (aU[b + 1] - T(2) * aP[b] + aU[b]) * sc.i4hh - (Fr - Fl) * sc.i2h;
       rP[q] = sTC[b] * rH[q] + (T(1) - sTC[b]) * RL;
     }
-    __syncthreads();
+    tile_sync<NT>();
   }
   const int gi = i0 + tid;
-  const bool own = gi < nx;
+  const bool own = tid < TX && gi < nx;
   T* Flim = A.limiter ? sFlim : sFH;
   T* Alim = A.limiter ? sAlim : sAH;
   for (int o = 0; o < A.nout; ++o) {
@@ -279,7 +305,7 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
           if (b >= H - 1) sULm[b] = u - m2 * (f - sFL[b - 1]);
         }
       }
-      __syncthreads();
+      tile_sync<NT>();
       // face factor 2 * parts (6 with diffusion, 2 without); the total face flux of the
       // form without double conservation takes factor 2 (the average is the mean of
       // u^{L,+} and u^{L,-}, one face correction each)
@@ -300,7 +326,7 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
           sAlim[b] = is_one(t) ? ah : al + t * (ah - al);
         }
       }
-      __syncthreads();
+      tile_sync<NT>();
     }
     if (own) {
       const int b = H + tid;
@@ -312,7 +338,7 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
       A.Oub[o][g] = ubo;
     }
     for (int q = 0; q < nq; ++q) {
-      const int gj = q == 0 ? gi : -1;   // point index j of u_{j+1/2}
+      const int gj = q == 0 && tid < TX ? gi : -1;   // point index j of u_{j+1/2}
       if (gj >= nx) continue;
       const size_t g = (size_t)(gj + poff);
       PT po;
@@ -326,7 +352,125 @@ __global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const
       }
       A.OV[o][g] = po;
     }
-    if (o + 1 < A.nout) __syncthreads();
+    if (o + 1 < A.nout) tile_sync<NT>();
+  }
+}
+
+// One CTA per 256-cell tile (4 CTAs per SM: 64 registers).
+template <int FLUX, class T, class PT>
+__global__ void __launch_bounds__(256, 4) stage1d_kernel(const DevModel m, const StageArgs2D<PT> A) {
+  using L = Tile1DLong;
+  __shared__ Shared1D<T, L::BX> sm;
+  const double dtv = *A.dt;
+  if (is_zero_bits(dtv)) return;   // uniform over the grid
+  stage1d_tile<FLUX, T, PT, L>(m, A, dtv, blockIdx.x * L::TX, threadIdx.x, sm);
+}
+
+// One warp per 26-cell tile, CTAs of one warp so that a short mesh spreads over the SMs.
+template <int FLUX, class T, class PT>
+__global__ void __launch_bounds__(32) stage1d_warp_kernel(const DevModel m, const StageArgs2D<PT> A) {
+  using L = Tile1DWarp;
+  __shared__ Shared1D<T, L::BX> sm;
+  const double dtv = *A.dt;
+  if (is_zero_bits(dtv)) return;   // uniform over the grid
+  stage1d_tile<FLUX, T, PT, L>(m, A, dtv, blockIdx.x * L::TX, threadIdx.x, sm);
+}
+
+// ---- whole steps of a short mesh in one launch
+//
+// A short mesh is bound by latency: as 5 launches per step (rate, step, 3 stages) a
+// 200-cell run took 59 us per step, most of it launch gaps, cold kernel starts and one
+// SM's FP64 unit. Here one cluster of 8 CTAs takes up to `nsteps` whole steps: warp w of
+// CTA r works on tile r + 8 w (26 cells), every stage ends in a cluster barrier (hardware,
+// no spinning), the CFL maximum is exchanged through distributed shared memory, and each
+// CTA forms the same step from it.
+template <int FLUX, class T, class PT>
+__global__ void __launch_bounds__(32 * MARCH_WARPS) march1d_kernel(const DevModel m,
+                                                                   const __grid_constant__ MarchArgs<PT> M) {
+  using L = Tile1DWarp;
+  __shared__ Shared1D<T, L::BX> sm[MARCH_WARPS];
+  __shared__ unsigned long long wbits[MARCH_WARPS];
+  __shared__ unsigned wflags[MARCH_WARPS];
+  __shared__ unsigned long long cbits[MARCH_CTAS];   // written by every CTA of the cluster
+  __shared__ unsigned cflags[MARCH_CTAS];
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int rank = (int)cl.block_rank(), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warps = blockDim.x >> 5;
+  const StageArgs2D<PT>& A0 = M.st[0];
+  const int nx = A0.nx, tile = rank + MARCH_CTAS * warp, i0 = tile * L::TX;
+  const bool has = i0 < nx;   // whole warp
+  double t = M.fin.t_acc ? *M.fin.t_acc : 0.0, dt = 0.0, steps = 0.0;
+  cl.sync();   // every CTA has started: its shared memory may be written
+  for (int n = 0; n < M.nsteps; ++n) {
+    if (M.dt_fixed > 0.0) {
+      dt = M.dt_fixed;
+    } else {
+      // the rate of this warp's cells (see dt_rate_maxu_kernel and dt_rate_kernel)
+      unsigned long long bits = 0ull;
+      unsigned flags = 0u;
+      const int i = i0 + lane;
+      if (has && lane < L::TX && i < nx) {
+        const double* ub = A0.ub;
+        const double u = ub[i], ih = M.fin.inv_h1, kd = M.fin.kmax * ih * ih;
+        auto rate = [&](double v) {
+          double d;
+          if constexpr (FLUX == FLUX_BL) d = bl_eval<double>(m, v).d[1];
+          else d = alpha_interval<FLUX, double>(m, 0, v, v);
+          return (unsigned long long)__double_as_longlong(d * ih + kd);
+        };
+        bits = rate(u);
+        if (A0.bc == AF_BC_DIRICHLET && (i == 0 || i == nx - 1)) {   // the end faces' ghosts (nx >= 4)
+          const unsigned long long e = rate(i == 0 ? A0.bc_left : A0.bc_right);
+          bits = e > bits ? e : bits;
+        }
+        if constexpr (FLUX == FLUX_BL) {
+          double un = ub[i + 1 == nx ? 0 : i + 1];
+          if (A0.bc != AF_BC_PERIODIC && i + 1 == nx) un = A0.bc == AF_BC_DIRICHLET ? A0.bc_right : u;
+          flags = crit_flags<FLUX>(m, 0, u, un);
+          if (A0.bc == AF_BC_DIRICHLET && i == 0) flags |= crit_flags<FLUX>(m, 0, A0.bc_left, u);
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, bits, o);
+        bits = v > bits ? v : bits;
+      }
+      flags = __reduce_or_sync(0xffffffffu, flags);
+      if (lane == 0) {
+        wbits[warp] = bits;
+        wflags[warp] = flags;
+      }
+      __syncthreads();
+      if (threadIdx.x < MARCH_CTAS) {
+        for (int w = 0; w < warps; ++w) {
+          bits = wbits[w] > bits ? wbits[w] : bits;
+          flags |= wflags[w];
+        }
+        // lane r stores this CTA's maximum into CTA r
+        cl.map_shared_rank(cbits, threadIdx.x)[rank] = bits;
+        cl.map_shared_rank(cflags, threadIdx.x)[rank] = flags;
+      }
+      cl.sync();
+      bits = 0ull;
+      flags = 0u;
+      for (int r = 0; r < MARCH_CTAS; ++r) {
+        bits = cbits[r] > bits ? cbits[r] : bits;
+        flags |= cflags[r];
+      }
+      dt = cfl_step(m, M.fin, bits, flags, t);
+      if (is_zero_bits(dt)) break;   // the end time is reached (uniform over the cluster)
+      if (dt > 0.0) steps += 1.0;
+    }
+    t += dt;
+    for (int k = 0; k < M.nstages; ++k) {
+      if (has) stage1d_tile<FLUX, T, PT, L>(m, M.st[k], dt, i0, lane, sm[warp]);
+      __syncwarp();
+      cl.sync();   // the stage's stores are visible to the cluster; also ends the reads of cbits
+    }
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    *M.fin.dt_out = dt;
+    if (M.fin.t_acc) *M.fin.t_acc = t;
+    if (M.fin.t_acc && M.fin.t_end > 0.0) *M.fin.count += steps;
   }
 }
 

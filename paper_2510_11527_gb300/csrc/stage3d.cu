@@ -595,34 +595,52 @@ cudaError_t launch_stage3d_f32(int flux, const DevModel& m, const StageArgs3D<fl
 
 // CFL rate of a 3D mesh: max over cells and directions of |f_l'(ub)| / h_l +
 // kappa_max / h_l^2 (the fluxes of 3D meshes have no interior extrema of f_l', so the
-// interval maximum over a face is taken at its end points, both cell averages)
+// interval maximum over a face is taken at its end points, both cell averages). |f_l'| is
+// a constant or a nondecreasing function of |u| and rounding is monotone, so it is the
+// rate at the largest |u|, reduced as a maximum of magnitude bits on the integer units
+// (zero and linear fluxes read nothing). The last block forms the step (dt_finish).
 template <int FLUX>
 __global__ void __launch_bounds__(RED_THREADS) rate3d_kernel(const DevModel m, size_t N, const double* __restrict__ ub,
                                                               double ih0, double ih1, double ih2, double kmax,
-                                                              unsigned long long* rate_bits) {
-  const double inv_h[3] = {ih0, ih1, ih2};
-  double best = 0.0;
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < N; q += (size_t)gridDim.x * blockDim.x) {
-    const double u = ub[q];
-    for (int l = 0; l < 3; ++l) best = tmax(best, dflux_abs<FLUX, double>(m, l, u) * inv_h[l] + kmax * inv_h[l] * inv_h[l]);
+                                                              unsigned long long* rate_bits, const DtFinal fin) {
+  unsigned long long mb = 0ull;
+  if constexpr (FLUX == FLUX_BURGERS) {
+    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < N; q += (size_t)gridDim.x * blockDim.x) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(ub[q]) & 0x7FFFFFFFFFFFFFFFull;
+      mb = b > mb ? b : mb;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long v = __shfl_xor_sync(0xffffffffu, mb, o);
+      mb = v > mb ? v : mb;
+    }
   }
-  for (int off = 16; off > 0; off >>= 1) best = tmax(best, __shfl_xor_sync(0xffffffffu, best, off));
-  if ((threadIdx.x & 31) == 0) atomicMax(rate_bits, (unsigned long long)__double_as_longlong(best));
+  __shared__ unsigned long long smb[RED_THREADS / 32];
+  if ((threadIdx.x & 31) == 0) smb[threadIdx.x >> 5] = mb;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < RED_THREADS / 32; ++w) mb = smb[w] > mb ? smb[w] : mb;
+    const double u = __longlong_as_double((long long)mb);
+    const double inv_h[3] = {ih0, ih1, ih2};
+    double best = 0.0;
+    for (int l = 0; l < 3; ++l) best = tmax(best, dflux_abs<FLUX, double>(m, l, u) * inv_h[l] + kmax * inv_h[l] * inv_h[l]);
+    atomicMax(rate_bits, (unsigned long long)__double_as_longlong(best));
+    dt_finish(rate_bits, m, fin);
+  }
 }
 
 cudaError_t launch_rate3d(int flux, const DevModel& m, const int* n, const double* ub, const double* inv_h, double kmax,
-                          unsigned long long* rate_bits, cudaStream_t s) {
-  const int blocks = 152 * 4;
+                          unsigned long long* rate_bits, const DtFinal& fin, int blocks, cudaStream_t s) {
   const size_t N = (size_t)n[0] * n[1] * n[2];
   switch (flux) {
     case FLUX_ZERO:
-      rate3d_kernel<FLUX_ZERO><<<blocks, RED_THREADS, 0, s>>>(m, N, ub, inv_h[0], inv_h[1], inv_h[2], kmax, rate_bits);
+      rate3d_kernel<FLUX_ZERO><<<1, RED_THREADS, 0, s>>>(m, N, ub, inv_h[0], inv_h[1], inv_h[2], kmax, rate_bits, fin);
       break;
     case FLUX_LINEAR:
-      rate3d_kernel<FLUX_LINEAR><<<blocks, RED_THREADS, 0, s>>>(m, N, ub, inv_h[0], inv_h[1], inv_h[2], kmax, rate_bits);
+      rate3d_kernel<FLUX_LINEAR><<<1, RED_THREADS, 0, s>>>(m, N, ub, inv_h[0], inv_h[1], inv_h[2], kmax, rate_bits, fin);
       break;
     case FLUX_BURGERS:
-      rate3d_kernel<FLUX_BURGERS><<<blocks, RED_THREADS, 0, s>>>(m, N, ub, inv_h[0], inv_h[1], inv_h[2], kmax, rate_bits);
+      rate3d_kernel<FLUX_BURGERS><<<blocks, RED_THREADS, 0, s>>>(m, N, ub, inv_h[0], inv_h[1], inv_h[2], kmax, rate_bits,
+                                                                 fin);
       break;
     default: return cudaErrorInvalidValue;
   }
