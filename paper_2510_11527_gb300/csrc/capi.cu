@@ -478,7 +478,8 @@ af_status af_create(const af_grid* grid, const af_flux* flux, const af_diff* dif
   // 3D: the FP64 averages and 7 point arrays per state, and 19 scratch arrays of the 3D
   // stage (sized for FP64)
   const size_t per_state = d3 ? al(c->n * 8) + 7 * al(c->n * ps) : al(ulen * 8) + 3 * al(plen * ps);
-  const size_t scr3 = d3 ? 19 * al(c->n * 8) : 0;
+  const bool scratch3 = d3 && opts->blend != AF_BLEND_OFF;   // the marching stage needs none
+  const size_t scr3 = scratch3 ? 19 * al(c->n * 8) : 0;
   const size_t scratch = al(8) * 2 + al(8 * 8) + al(8 * af::RED_MAX_BLOCKS) + al(8) + al(sizeof(DevStats)) + al(c->n * 8);
   const size_t total = per_state * c->nbuf + scratch + scr3;
   if (cudaMalloc(&c->block, total) != cudaSuccess) {
@@ -508,7 +509,7 @@ af_status af_create(const af_grid* grid, const af_flux* flux, const af_diff* dif
   c->rate_bits = (unsigned long long*)p; p += al(24);
   c->stats = (DevStats*)p; p += al(sizeof(DevStats));
   c->s_ext = (double*)p; p += al(c->n * 8);
-  for (int k = 0; d3 && k < 19; ++k) { c->scr3[k] = p; p += al(c->n * 8); }
+  for (int k = 0; scratch3 && k < 19; ++k) { c->scr3[k] = p; p += al(c->n * 8); }
   if (cudaMemset(c->block, 0, total) != cudaSuccess || cudaMallocHost(&c->host_pinned, 8 * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(c->block);

@@ -27,8 +27,9 @@ namespace af {
 // by 256 threads for long meshes, and 26 cells by one warp (halo included, one box
 // position per lane) for meshes that would otherwise leave most SMs idle: GB300's FP64
 // unit passes 2 lanes per clock and SM, so a short mesh is bound by the FP64 rate of the
-// few SMs it runs on (200 cells in one 256-cell tile: 17 us per stage, bound by one SM's
-// FP64 unit; 8 one-warp tiles on 8 SMs: see march1d_kernel).
+// few SMs it runs on. Launched steps of Example 6.5's problem, FP64, 256-cell tiles /
+// one-warp tiles: 200 cells 57 / 43 us, 10,000 61 / 43 us, 38,000 66 / 49 us; beyond
+// 152 x 256 cells the long tile, whose halo costs 2 % of the work instead of 23 %.
 template <int TX_, int NT_>
 struct Tile1D {
   static constexpr int TX = TX_, NT = NT_, H = 3, BX = TX + 2 * H;
@@ -376,14 +377,15 @@ __global__ void __launch_bounds__(32) stage1d_warp_kernel(const DevModel m, cons
   stage1d_tile<FLUX, T, PT, L>(m, A, dtv, blockIdx.x * L::TX, threadIdx.x, sm);
 }
 
-// ---- whole steps of a short mesh in one launch
+// Whole steps of a short mesh in one launch.
 //
-// A short mesh is bound by latency: as 5 launches per step (rate, step, 3 stages) a
-// 200-cell run took 59 us per step, most of it launch gaps, cold kernel starts and one
-// SM's FP64 unit. Here one cluster of 8 CTAs takes up to `nsteps` whole steps: warp w of
-// CTA r works on tile r + 8 w (26 cells), every stage ends in a cluster barrier (hardware,
-// no spinning), the CFL maximum is exchanged through distributed shared memory, and each
-// CTA forms the same step from it.
+// A short mesh is bound by latency: as 5 launches per step (rate, step size, 3 stages) a
+// 200-cell FP64 run took 59 us per step, launch gaps and one SM's FP64 unit. Here one
+// cluster of 8 CTAs takes up to `nsteps` whole steps: warp w of CTA r works on tile
+// r + 8 w (26 cells), every stage ends in a cluster barrier (hardware, no spinning), the
+// CFL maximum is exchanged through distributed shared memory, and each CTA forms the same
+// step from it: 31 us per step, now the chain of ~1300 instructions of one tile per stage.
+// Up to 832 cells a step costs the same; launched stages of one-warp tiles take 43 us.
 template <int FLUX, class T, class PT>
 __global__ void __launch_bounds__(32 * MARCH_WARPS) march1d_kernel(const DevModel m,
                                                                    const __grid_constant__ MarchArgs<PT> M) {

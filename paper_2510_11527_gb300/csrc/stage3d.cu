@@ -200,108 +200,6 @@ __global__ void __launch_bounds__(T3) limit3d_kernel(const DevModel m, const Sta
   }
 }
 
-template <int FLUX, class T>
-__global__ void __launch_bounds__(T3) update3d_kernel(const DevModel m, const StageArgs3D<T> A, int o) {
-  const double dtv = *A.dt;
-  if (dtv == 0.0) return;   // uniform over the grid
-  const double tau = A.tcoef[o] * dtv;
-  const double cA = A.cA[o], cF = A.cF[o];
-  // mu_l = tau / h_l and nu_l = tau / h_l^2 of this launch, once per block
-  __shared__ double sMu[3], sNu[3];
-  if (threadIdx.x < 3) {
-    const int l = threadIdx.x;
-    sMu[l] = tau * A.inv_h[l];
-    sNu[l] = sMu[l] * A.inv_h[l];
-  }
-  __syncthreads();
-  const size_t N = cells3(A);
-  const T taut = T(tau), cAt = T(cA), cFt = T(cF), umin = T(m.umin), umax = T(m.umax), g = T(A.gamma);
-  // an integer test: GB300 runs FP64 compares on its slow FP64 unit
-  const bool comb = !is_zero_bits(cA);
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < N; q += (size_t)gridDim.x * blockDim.x) {
-    int c[3];
-    decode3(A, q, c);
-    const FineAxes fa = fine_axes(A, c);
-    // limited cell-average update (eq. multid_limited_average), in FP64
-    double v = A.ub[q];
-    for (int l = 0; l < 3; ++l) {
-      const double mu = sMu[l], nu = sNu[l];
-      const size_t qm = nbr3(A, c, l, -1), qp = nbr3(A, c, l, 1);
-      const double f0 = wide(A.Flim[l][q]), fm = wide(A.Flim[l][qm]);
-      const double a0 = wide(A.Alim[l][q]), am = wide(A.Alim[l][qm]), ap = wide(A.Alim[l][qp]);
-      v = v - mu * (f0 - fm) + nu * (ap - 2.0 * a0 + am);
-    }
-    double ubo = comb ? rk_comb(cA, A.Aub[o][q], cF, v) : rk_scale(cF, v);
-    if (A.limiter && A.sg[o]) ubo = safeguard<double>(ubo, m.umin, m.umax, A.tol, A.stats, true);
-    A.Oub[o][q] = ubo;
-    // point values owned by the cell: kinds 1..7 at fine 2c + s
-    for (int s = 1; s < 8; ++s) {
-      const int p[3] = {s & 1, (s >> 1) & 1, (s >> 2) & 1};   // offsets from 2c
-      T acc = T(0);
-      for (int l = 0; l < 3; ++l) {
-        const T ih = A.inv_hT[l];
-        T z[5], fz[5], dz[5], az[5];
-        for (int t = 0; t < 5; ++t) {
-          int f[3] = {p[0], p[1], p[2]};
-          f[l] += t - 2;
-          z[t] = zoff(A, fa, f[0], f[1], f[2]);
-          fz[t] = flux<FLUX, T>(m, l, z[t]);
-          dz[t] = dflux_abs<FLUX, T>(m, l, z[t]);
-          az[t] = apot<T>(m, z[t]);
-        }
-        T rh;
-        if constexpr (FLUX == FLUX_ZERO) {
-          // the diffusion part of line_res alone (its convection part is an exact zero)
-          rh = (T(16) * (az[1] + az[3]) - (az[0] + az[4]) - T(30) * az[2]) * A.i3h2T[l];
-        } else {
-          const T alpha = tmax(tmax(tmax(dz[0], dz[1]), tmax(dz[3], dz[4])), dz[2]);
-          rh = line_res<T>(z[0], z[1], z[2], z[3], z[4], fz[0], fz[1], fz[3], fz[4], alpha, az[0], az[1], az[2], az[3],
-                           az[4], A.i6hT[l], A.i3h2T[l]);
-        }
-        T r = rh;
-        if (A.blend) {
-          // weight: min of theta^{c,s}_l over the l-faces holding the point (s_l = 1),
-          // else of theta^{d,s}_l over the cells holding it
-          const bool onface = (s >> l) & 1;
-          T w = T(2);
-          for (int bits = 0; bits < 8; ++bits) {
-            int cc[3] = {c[0], c[1], c[2]};
-            bool ok = true;
-            for (int t = 0; t < 3; ++t) {
-              if (!((bits >> t) & 1)) continue;
-              if (t == l || !((s >> t) & 1)) { ok = false; break; }
-              cc[t] = cc[t] + 1 == A.n[t] ? 0 : cc[t] + 1;   // periodic, so nbr3 below sees wrapped coordinates
-            }
-            if (!ok) continue;
-            const size_t qq = cell3(A, cc);
-            const T sv = A.S[l][qq];
-            const T wv = onface ? exp(-g * (T(0.5) * (sv + A.S[l][nbr3(A, cc, l, 1)]))) : exp(-g * sv);
-            w = (w == T(2)) ? wv : tmin(w, wv);
-          }
-          // low-order residual on the +-h/2 neighbours (a centre replaced by its average)
-          int fm[3] = {p[0], p[1], p[2]}, fp[3] = {p[0], p[1], p[2]};
-          fm[l] -= 1;
-          fp[l] += 1;
-          const T zm = zoff(A, fa, fm[0], fm[1], fm[2], true), z0 = z[2],
-                  zp = zoff(A, fa, fp[0], fp[1], fp[2], true);
-          const T Fr = T(0.5) * (flux<FLUX, T>(m, l, z0) + flux<FLUX, T>(m, l, zp)) -
-                       T(0.5) * alpha_interval<FLUX, T>(m, l, z0, zp) * (zp - z0);
-          const T Fl = T(0.5) * (flux<FLUX, T>(m, l, zm) + flux<FLUX, T>(m, l, z0)) -
-                       T(0.5) * alpha_interval<FLUX, T>(m, l, zm, z0) * (z0 - zm);
-          const T RL = (apot<T>(m, zp) - T(2) * apot<T>(m, z0) + apot<T>(m, zm)) * (T(4) * ih * ih) - (Fr - Fl) * (T(2) * ih);
-          r = w * rh + (T(1) - w) * RL;
-        }
-        acc = (l == 0) ? r : acc + r;
-      }
-      T pv = A.pt[s][q] + taut * acc;
-      if (A.limiter) pv = tmin(tmax(pv, umin), umax);
-      T po = comb ? rk_comb(cAt, A.Apt[o][s][q], cFt, pv) : rk_scale(cFt, pv);
-      if (A.limiter && A.sg[o]) po = safeguard<T>(po, umin, umax, A.tol, A.stats);
-      A.Opt[o][s][q] = po;
-    }
-  }
-}
-
 // K4 with the point values staged: one CTA per tile of U3X x U3Y x U3Z cells loads the
 // centres and the 7 point kinds of the tile and a one-cell halo into shared memory
 // once, with a(z) evaluated once per location; every 5-point line of the tile's points
@@ -586,10 +484,13 @@ cudaError_t dispatch3d(int flux, const DevModel& m, const StageArgs3D<T>& a, cud
 
 }  // namespace
 
+// without the blend one marching launch per output (march3d.cuh); with it the four kernels
 cudaError_t launch_stage3d_f64(int flux, const DevModel& m, const StageArgs3D<double>& a, cudaStream_t s) {
+  if (!a.blend) return launch_march3d_f64(flux, m, a, s);
   return dispatch3d<double>(flux, m, a, s);
 }
 cudaError_t launch_stage3d_f32(int flux, const DevModel& m, const StageArgs3D<float>& a, cudaStream_t s) {
+  if (!a.blend) return launch_march3d_f32(flux, m, a, s);
   return dispatch3d<float>(flux, m, a, s);
 }
 
