@@ -11,6 +11,7 @@
 
 #include "af.h"
 #include "launch.h"
+#include "march3d_plan.h"
 #include "model_host.h"
 #include "reduce.cuh"
 #include "state_io.cuh"
@@ -478,7 +479,9 @@ af_status af_create(const af_grid* grid, const af_flux* flux, const af_diff* dif
   // 3D: the FP64 averages and 7 point arrays per state, and 19 scratch arrays of the 3D
   // stage (sized for FP64)
   const size_t per_state = d3 ? al(c->n * 8) + 7 * al(c->n * ps) : al(ulen * 8) + 3 * al(plen * ps);
-  const bool scratch3 = d3 && opts->blend != AF_BLEND_OFF;   // the marching stage needs none
+  const int n3[3] = {c->nx, c->ny, c->nz};
+  // the marching 3D stage needs no scratch arrays
+  const bool scratch3 = d3 && (opts->blend != AF_BLEND_OFF || !af::march3d_takes(flux->kind, c->prec == AF_PREC_FP64, n3));
   const size_t scr3 = scratch3 ? 19 * al(c->n * 8) : 0;
   const size_t scratch = al(8) * 2 + al(8 * 8) + al(8 * af::RED_MAX_BLOCKS) + al(8) + al(sizeof(DevStats)) + al(c->n * 8);
   const size_t total = per_state * c->nbuf + scratch + scr3;

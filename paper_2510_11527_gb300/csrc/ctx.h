@@ -28,7 +28,7 @@ struct af_ctx {
   int nz = 1;
   double dz = 1, inv_h3 = 0;
   void* k3[4][8] = {};                // [b][0]: FP64 averages; [b][1..7]: points (FP64 or FP32)
-  void* scr3[19] = {};                // stencil precision (with the blend only)
+  void* scr3[19] = {};                // stencil precision (the four-kernel stage only)
   size_t pn = 0;                      // pnx * pny entries per device array (1D: max(n, np))
   double dx = 1, dy = 1, inv_h1 = 1, inv_h2 = 1, kmax = 0, cfl = 0.165, cfl_diff = 0, tol = 0;
   bool bounds_pending = false;

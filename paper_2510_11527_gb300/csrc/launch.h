@@ -37,8 +37,8 @@ cudaError_t launch_stage2d_rect_f32(int flux, bool blend, const DevModel& m, con
                                     cudaStream_t s);
 cudaError_t launch_stage3d_f64(int flux, const DevModel& m, const StageArgs3D<double>& a, cudaStream_t s);
 cudaError_t launch_stage3d_f32(int flux, const DevModel& m, const StageArgs3D<float>& a, cudaStream_t s);
-// the 3D stage without the blend (march3d.cuh)
-cudaError_t launch_march3d_f64(int flux, const DevModel& m, const StageArgs3D<double>& a, cudaStream_t s);
+// the marching 3D stage (march3d.cuh; FP64: the zero flux)
+cudaError_t launch_march3d_f64(const DevModel& m, const StageArgs3D<double>& a, cudaStream_t s);
 cudaError_t launch_march3d_f32(int flux, const DevModel& m, const StageArgs3D<float>& a, cudaStream_t s);
 cudaError_t launch_rate3d(int flux, const DevModel& m, const int* n, const double* ub, const double* inv_h, double kmax,
                           unsigned long long* rate_bits, const DtFinal& fin, int blocks, cudaStream_t s);

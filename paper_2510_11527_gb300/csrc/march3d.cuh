@@ -24,29 +24,18 @@
 // with compensation, so the increment carries about 46 bits; it is widened once and added
 // to the FP64 average.
 //
-// Measured (porous medium; the four kernels with 19 scratch arrays that this replaces,
-// which the blend still takes): FP32-mixed 128^3 SSP-RK3 step 1.90 -> 0.50 ms, FP64 80^3
+// Measured (porous medium; against the four kernels with 19 scratch arrays, which the blend
+// and, where they are faster, FP64 meshes still take: march3d_takes): FP32-mixed 128^3 SSP-RK3 step 1.90 -> 0.50 ms, FP64 80^3
 // SSP-RK(5,4) step 3.36 -> 2.55 ms. FP64 is bound by the FP64 unit (77 % of its cycles
 // busy), FP32-mixed by instruction issue (about 900 instructions per layer and full row)
 // and the waits of one CTA's 16 warps on each other at the barrier; DRAM moves 58 bytes
 // per cell and stage. With two barriers per step the FP32 step took 0.66 ms.
 #pragma once
 #include "launch.h"
+#include "march3d_plan.h"
 #include "stencil.cuh"
 
 namespace af {
-
-constexpr int M3_BAND = 28;   // output columns per tile
-
-// Rows per CTA. The CTA's registers are the SM's: 16 rows at 128, 12 at 168 and 8 at 255
-// registers per thread; more rows cost fewer halo rows per output row, fewer registers
-// spill (FP64 with a flux at 12 rows: 0.9 KB per thread; porous medium 80^3 FP64 at 8 / 12
-// rows: 2.85 / 2.67 ms per SSP-RK(5,4) step).
-template <int FLUX, class T>
-constexpr int m3_rows() {
-  if (sizeof(T) == 8) return FLUX == FLUX_ZERO ? 12 : 8;
-  return FLUX == FLUX_ZERO ? 16 : 12;
-}
 
 // the launch's scalars
 template <class T>
@@ -278,9 +267,8 @@ __device__ __forceinline__ void m3_limit(const DevModel& m, const M3Scal<T>& k, 
 // three layers are kept) and, one step later, its centres' potentials and its y-limiter's
 // results (two steps). With that one barrier per step is enough: a slot is written again
 // only after a barrier that every reader of its last contents has passed.
-template <int FLUX, class T>
+template <int FLUX, class T, int TY>
 struct M3Shared {
-  static constexpr int TY = m3_rows<FLUX, T>();
   static constexpr int NA = 7 + 1 + (FLUX == FLUX_ZERO ? 4 : 7);   // a of kinds 1 .. 7, U, z
   static constexpr int NB = FLUX == FLUX_ZERO ? 2 : 4;             // a(C), A_y limited [, C, F_y limited]
   T a[3][NA][TY][32];
@@ -292,11 +280,10 @@ struct M3Shared {
   }
 };
 
-template <int FLUX, int DIFF, class T>
-__global__ void __launch_bounds__(32 * m3_rows<FLUX, T>(), 1)
+template <int FLUX, int DIFF, class T, int TY>
+__global__ void __launch_bounds__(32 * TY, 1)
     march3d_kernel(const DevModel m, const __grid_constant__ StageArgs3D<T> A, int o, int S, int bands, int rows) {
-  using SH = M3Shared<FLUX, T>;
-  constexpr int TY = SH::TY;
+  using SH = M3Shared<FLUX, T, TY>;
   constexpr bool CONV = FLUX != FLUX_ZERO;
   extern __shared__ __align__(16) unsigned char m3_raw[];
   SH& sh = *reinterpret_cast<SH*>(m3_raw);
@@ -343,10 +330,12 @@ __global__ void __launch_bounds__(32 * m3_rows<FLUX, T>(), 1)
   for (int r = zs - 2; r <= ze + 1; ++r) {
     const int par = r & 1;
     U = to_stencil<T>(un);
+    // of the last layer only the averages are read (in FP32 the test costs more than it saves)
+    const bool pts = sizeof(T) == 4 || r <= ze;
 #pragma unroll
     for (int s = 1; s < 8; ++s) {
       z[s] = pn[s];
-      a[s] = apot_k<DIFF, T>(m, z[s]);
+      if (pts) a[s] = apot_k<DIFF, T>(m, z[s]);
     }
     const unsigned qc = q;
     // next layer
@@ -397,7 +386,7 @@ __global__ void __launch_bounds__(32 * m3_rows<FLUX, T>(), 1)
     T AHx = T(0), AHz = T(0), FHx = T(0), FHz = T(0), Fy = T(0), Ay = T(0);
     T am2, am3, am6, am7, zm2, zm3, zm6, zm7;   // row below
     const T a1x = shup(a[1]), a3x = shup(a[3]), a5x = shup(a[5]), a7x = shup(a[7]);   // column before
-    if (mid) {
+    if (mid && pts) {
       am2 = sh.a[ca][1][rm][lane];
       am3 = sh.a[ca][2][rm][lane];
       am6 = sh.a[ca][5][rm][lane];
@@ -406,7 +395,7 @@ __global__ void __launch_bounds__(32 * m3_rows<FLUX, T>(), 1)
       zm3 = sh.a[ca][SH::zslot(3)][rm][lane];
       zm6 = sh.a[ca][SH::zslot(6)][rm][lane];
       zm7 = sh.a[ca][SH::zslot(7)][rm][lane];
-      T AHy, FHy = T(0);
+      T AHy = T(0), FHy = T(0);
       if constexpr (sizeof(T) == 4) {
         // the layer's plane of centres (kinds 0 .. 3) and its upper plane of z-faces (4 .. 7)
         // as 3 x 3 locations around the cell, index 3 (my + 1) + mx + 1
@@ -497,8 +486,11 @@ __global__ void __launch_bounds__(32 * m3_rows<FLUX, T>(), 1)
         const T e1 = shup(z[1]) + z[1], e2 = zm2 + z[2], e3 = shup(y3) + y3;
         const T e5 = shup(z[5]) + z[5], e6 = zm6 + z[6], e7 = shup(y7) + y7;
         const T fsum = e1 + e2 + (lv.z[0] + z[4]), esum = e3 + (lv.z[1] + e5) + (lv.z[2] + e6);
-        z[0] = sfma(T(216), U, -sfma(T(16), fsum, sfma(T(4), esum, lv.z[3] + e7))) * T(1.0 / 64.0);
-        a[0] = apot_k<DIFF, T>(m, z[0]);
+        const bool whole = r > zs - 2;   // the first layer only leaves its upper plane
+        if (whole) {
+          z[0] = sfma(T(216), U, -sfma(T(16), fsum, sfma(T(4), esum, lv.z[3] + e7))) * T(1.0 / 64.0);
+          a[0] = apot_k<DIFF, T>(m, z[0]);
+        }
         lv.z[0] = z[4];
         lv.z[1] = e5;
         lv.z[2] = e6;
@@ -512,10 +504,12 @@ __global__ void __launch_bounds__(32 * m3_rows<FLUX, T>(), 1)
         lv.a[1] = b5;
         lv.a[2] = b6;
         lv.a[3] = b7;
-        const T c16 = T(16) * a[0], r216 = T(1.0 / 216.0);
-        AHx = sfma(T(8), c16 + sfma(T(4), b2 + Fz, Eyz), -sfma(T(16), b1, sfma(T(4), b3 + Exz, V))) * r216;
-        AHy = sfma(T(8), c16 + sfma(T(4), b1 + Fz, Exz), -sfma(T(16), b2, sfma(T(4), b3 + Eyz, V))) * r216;
-        AHz = sfma(T(8), c16 + sfma(T(4), b1 + b2, b3), -sfma(T(16), Fz, sfma(T(4), Exz + Eyz, V))) * r216;
+        if (whole) {
+          const T r216 = T(1.0 / 216.0);
+          AHx = sfma(T(8), sfma(T(16), a[0], sfma(T(4), b2 + Fz, Eyz)), -sfma(T(16), b1, sfma(T(4), b3 + Exz, V))) * r216;
+          AHy = sfma(T(8), sfma(T(16), a[0], sfma(T(4), b1 + Fz, Exz)), -sfma(T(16), b2, sfma(T(4), b3 + Eyz, V))) * r216;
+          AHz = sfma(T(8), sfma(T(16), a[0], sfma(T(4), b1 + b2, b3)), -sfma(T(16), Fz, sfma(T(4), Exz + Eyz, V))) * r216;
+        }
         if constexpr (CONV) {
           // Simpson averages of f_l over the upper faces
           auto f = [&](int l, T v) { return flux<FLUX, T>(m, l, v); };
@@ -667,40 +661,31 @@ __global__ void __launch_bounds__(32 * m3_rows<FLUX, T>(), 1)
 
 // ---- launch (host)
 
-// Layers per strip: the number of strips with the fewest steps over all waves of CTAs
-// (one CTA per SM; a strip repeats about 3 steps' work of warm-up and drain).
-static int m3_strip(int nz, long long tiles) {
-  long long best = -1;
-  int S = nz;
-  for (int s = 1; s <= nz && s <= 152 * 8; ++s) {
-    const int L = (nz + s - 1) / s;
-    const long long waves = (tiles * ((nz + L - 1) / L) + 151) / 152;
-    const long long cost = waves * (L + 3);
-    if (best < 0 || cost < best) {
-      best = cost;
-      S = L;
-    }
-  }
-  return S;
-}
-
-template <int FLUX, int DIFF, class T>
-static cudaError_t march3d_go(const DevModel& m, const StageArgs3D<T>& a, cudaStream_t s) {
-  constexpr int TY = m3_rows<FLUX, T>();
-  const int bands = (a.n[0] + M3_BAND - 1) / M3_BAND, rows = (a.n[1] + TY - 5) / (TY - 4);
-  const int S = m3_strip(a.n[2], (long long)bands * rows);
-  const long long blocks = (long long)bands * rows * ((a.n[2] + S - 1) / S);
+template <int FLUX, int DIFF, class T, int TY>
+static cudaError_t march3d_rows(const DevModel& m, const StageArgs3D<T>& a, const M3Plan& p, cudaStream_t s) {
+  const long long blocks = (long long)p.bands * p.rows * ((a.n[2] + p.S - 1) / p.S);
   if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-  auto kern = march3d_kernel<FLUX, DIFF, T>;
-  const int smem = (int)sizeof(M3Shared<FLUX, T>);
+  auto kern = march3d_kernel<FLUX, DIFF, T, TY>;
+  const int smem = (int)sizeof(M3Shared<FLUX, T, TY>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   for (int o = 0; o < a.nout; ++o) {
-    kern<<<(unsigned)blocks, 32 * TY, smem, s>>>(m, a, o, S, bands, rows);
+    kern<<<(unsigned)blocks, 32 * TY, smem, s>>>(m, a, o, p.S, p.bands, p.rows);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+template <int FLUX, int DIFF, class T>
+static cudaError_t march3d_go(const DevModel& m, const StageArgs3D<T>& a, cudaStream_t s) {
+  constexpr int TY = m3_rows(FLUX, sizeof(T) == 8);
+  const M3Plan p = m3_plan(a.n, TY);
+  if constexpr (TY > M3_ROWS_SMALL) {
+    const M3Plan q = m3_plan(a.n, M3_ROWS_SMALL);
+    if (q.cost < p.cost) return march3d_rows<FLUX, DIFF, T, M3_ROWS_SMALL>(m, a, q, s);
+  }
+  return march3d_rows<FLUX, DIFF, T, TY>(m, a, p, s);
 }
 
 template <int FLUX, class T>
@@ -708,16 +693,6 @@ static cudaError_t march3d_diff(const DevModel& m, const StageArgs3D<T>& a, cuda
   if (m.diff_kind == AF_DIFF_CONST) return march3d_go<FLUX, DK_CONST, T>(m, a, s);
   if (m.diff_kind == AF_DIFF_PME && m.pme_e == 2) return march3d_go<FLUX, DK_PME2, T>(m, a, s);
   return march3d_go<FLUX, DK_GENERIC, T>(m, a, s);
-}
-
-template <class T>
-static cudaError_t march3d_flux(int flux, const DevModel& m, const StageArgs3D<T>& a, cudaStream_t s) {
-  switch (flux) {
-    case FLUX_ZERO: return march3d_diff<FLUX_ZERO, T>(m, a, s);
-    case FLUX_LINEAR: return march3d_diff<FLUX_LINEAR, T>(m, a, s);
-    case FLUX_BURGERS: return march3d_diff<FLUX_BURGERS, T>(m, a, s);
-    default: return cudaErrorInvalidValue;
-  }
 }
 
 }  // namespace af

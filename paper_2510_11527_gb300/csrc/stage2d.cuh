@@ -84,10 +84,11 @@ template <class T> struct PointStore<FLUX_BL, T> {
   static constexpr int NQ = DOFF + 3, NQU = NQ;
 };
 
-template <int FLUX, class T, bool BLEND, int TX_ = 32, int TY_ = 8>
+template <int FLUX, class T, bool BLEND, int TX_ = 32, int TY_ = 8, int NT_ = TX_ * TY_>
 struct Tile2D {
-  static constexpr int TX = TX_, TY = TY_, NT = TX * TY;
-  static_assert(NT == 256, "stage tiles use 256 threads");
+  static constexpr int TX = TX_, TY = TY_, NT = NT_;
+  static_assert(NT % 32 == 0 && NT >= 64 && NT >= TX * TY && TX % 2 == 0,
+                "whole warps, one per output; a thread per cell; paired loads");
   static constexpr int H = BLEND ? 3 : 2;
   static constexpr int BX = TX + 2 * H, BY = TY + 2 * H, BN = BX * BY;
   static constexpr int NQ = PointStore<FLUX, T>::NQ, NQU = PointStore<FLUX, T>::NQU;
@@ -192,10 +193,11 @@ __device__ __forceinline__ int rect_face(int I, int n) {
 // PAIRED enables the paired vector loads of interior halo boxes (P0). RECT selects a 2D
 // rectangle with outflow ends in its padded layout (reflected ghost loads, masked stores);
 // periodic meshes compile without any of it.
-template <int FLUX, class T, class PT, bool BLEND, int TX_ = 32, int TY_ = 8, bool PAIRED = true, bool RECT = false>
+template <int FLUX, class T, class PT, bool BLEND, int TX_ = 32, int TY_ = 8, bool PAIRED = true, bool RECT = false,
+          int NT_ = TX_ * TY_>
 __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<PT>& A, const int i0, const int j0,
                                            unsigned char* smem_raw) {
-  using L = Tile2D<FLUX, T, BLEND, TX_, TY_>;
+  using L = Tile2D<FLUX, T, BLEND, TX_, TY_, NT_>;
   using PS = PointStore<FLUX, T>;
   constexpr int TX = L::TX, TY = L::TY, NT = L::NT, H = L::H, BX = L::BX, BY = L::BY, BN = L::BN;
   constexpr int NQ = L::NQ;
@@ -481,13 +483,16 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
   };
   constexpr int tV = 0, tX = 1, tY = 2, tC = 3;
   const int bo = (ty + H) * BX + (tx + H);   // own box index
-  T rV1, rV2, rX1, rX2, rY1, rY2;
+  const bool cell = NT == TX * TY || tid < TX * TY;   // a thread with a cell of its own
+  T rV1 = T(0), rV2 = T(0), rX1 = T(0), rX2 = T(0), rY1 = T(0), rY2 = T(0);
+  if (cell) {
   rV1 = line(0, tV, bo - 1, tY, bo, tV, bo, tY, bo + 1, tV, bo + 1);
   rV2 = line(1, tV, bo - BX, tX, bo, tV, bo, tX, bo + BX, tV, bo + BX);
   rX1 = line(0, tX, bo - 1, tC, bo, tX, bo, tC, bo + 1, tX, bo + 1);
   rX2 = line(1, tX, bo - BX, tV, bo - BX, tX, bo, tV, bo, tX, bo + BX);
   rY1 = line(0, tY, bo - 1, tV, bo - 1, tY, bo, tV, bo, tY, bo + 1);
   rY2 = line(1, tY, bo - BX, tC, bo, tY, bo, tC, bo + BX, tY, bo + BX);
+  }
 
   T* sFH1 = arr(L::A_FH1);
   T* sFH2 = arr(L::A_FH2);
@@ -628,7 +633,7 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
                    T(0.5) * alpha_interval_pre<FLUX, T>(m, dir, pm.z, p0.z, pm.d, p0.d) * (p0.z - pm.z);
       return (pp.a - T(2) * p0.a + pm.a) * (dir == 0 ? i4h21 : i4h22) - (Fr - Fl) * (dir == 0 ? i2h1 : i2h2);
     };
-    const int b = bo;
+    const int b = cell ? bo : H * BX + H;
     const T LV1 = lowres(0, pt(tY, b, 0), pt(tV, b, 0), pt(tY, b + 1, 0));
     const T LV2 = lowres(1, pt(tX, b, 1), pt(tV, b, 1), pt(tX, b + BX, 1));
     const T LX1 = lowres(0, cu(b, 0), pt(tX, b, 0), cu(b + 1, 0));
@@ -650,7 +655,7 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
 
   // ---- per output: low-order states, limiter, update ------------------------------------
   const int gi = i0 + tx, gj = j0 + ty;
-  const bool own = gi < nx && gj < ny;
+  const bool own = cell && gi < nx && gj < ny;
   const size_t g = (size_t)gj * nx + gi;
   T* sULp1 = arr(L::A_ULP1);
   T* sULm1 = arr(L::A_ULM1);
@@ -800,12 +805,12 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
   }
 }
 
-// One CTA per 32 x 8 tile of a single mesh (row-major tile index in blockIdx.x).
-template <int FLUX, class T, class PT, bool BLEND, bool RECT = false>
-__global__ void __launch_bounds__(256) stage2d_kernel(const DevModel m, const StageArgs2D<PT> A) {
+// One CTA per TX x TY tile of a single mesh (row-major tile index in blockIdx.x).
+template <int FLUX, class T, class PT, bool BLEND, bool RECT = false, int TX = 32, int TY = 8, int NT = TX * TY>
+__global__ void __launch_bounds__(NT) stage2d_kernel(const DevModel m, const StageArgs2D<PT> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int tiles_x = (A.nx + 31) / 32, t = blockIdx.x;   // 1D grid: no 65535 limit on rows
-  stage_tile<FLUX, T, PT, BLEND, 32, 8, true, RECT>(m, A, (t % tiles_x) * 32, (t / tiles_x) * 8, smem_raw);
+  const int tiles_x = (A.nx + TX - 1) / TX, t = blockIdx.x;   // 1D grid: no 65535 limit on rows
+  stage_tile<FLUX, T, PT, BLEND, TX, TY, true, RECT, NT>(m, A, (t % tiles_x) * TX, (t / tiles_x) * TY, smem_raw);
 }
 
 // The same for the FP32 stencils without the blend, compiled for 6 resident CTAs per SM

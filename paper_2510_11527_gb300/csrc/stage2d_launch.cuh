@@ -13,29 +13,53 @@
 
 namespace af {
 
-template <int FLUX, class T, bool BLEND, bool RECT>
+template <int FLUX, class T, bool BLEND, bool RECT, int TX, int TY, int NT>
 static auto stage2d_kernel_for() {
-  if constexpr (std::is_same_v<T, float> && !BLEND) return stage2d_kernel_f32occ6<FLUX, RECT>;
-  else return stage2d_kernel<FLUX, T, T, BLEND, RECT>;
+  if constexpr (std::is_same_v<T, float> && !BLEND && TX == 32) return stage2d_kernel_f32occ6<FLUX, RECT>;
+  else return stage2d_kernel<FLUX, T, T, BLEND, RECT, TX, TY, NT>;
 }
 
-template <int FLUX, class T, bool BLEND, bool RECT>
-static cudaError_t stage2d_go(const DevModel& m, const StageArgs2D<T>& a, cudaStream_t s) {
-  if constexpr (std::is_same_v<T, float> && !RECT)
-    return launch_stream2d_f32(FLUX, BLEND ? (a.blend_external ? 2 : 1) : 0, m, a, s);
-  using L = Tile2D<FLUX, T, BLEND>;
+// Work of a mesh's busiest SM with TX x TY tiles of halo H, in warps of box positions:
+// tiles dealt to 152 SMs, each worth its box (what the FP64 unit of an SM spends on a
+// tile; on a short mesh also the length of a CTA's phases).
+inline long long tile_cost(int nx, int ny, int TX, int TY, int H) {
+  const long long tiles = (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
+  return (tiles + 151) / 152 * (((TX + 2 * H) * (TY + 2 * H) + 31) / 32);
+}
+
+template <int FLUX, class T, bool BLEND, bool RECT, int TX, int TY, int NT = TX * TY>
+static cudaError_t stage2d_tiles(const DevModel& m, const StageArgs2D<T>& a, cudaStream_t s) {
+  using L = Tile2D<FLUX, T, BLEND, TX, TY, NT>;
   static bool attr = false;
-  auto k = stage2d_kernel_for<FLUX, T, BLEND, RECT>();
+  auto k = stage2d_kernel_for<FLUX, T, BLEND, RECT, TX, TY, NT>();
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::SMEM);
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  const long long tiles = (long long)((a.nx + L::TX - 1) / L::TX) * ((a.ny + L::TY - 1) / L::TY);
+  const long long tiles = (long long)((a.nx + TX - 1) / TX) * ((a.ny + TY - 1) / TY);
   if (tiles > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-  dim3 grid((unsigned)tiles);
-  k<<<grid, L::NT, L::SMEM, s>>>(m, a);
+  k<<<(unsigned)tiles, L::NT, L::SMEM, s>>>(m, a);
   return cudaGetLastError();
+}
+
+// Tile shape by mesh: 32 x 8 on large meshes (its halo box is 1.7 times the tile), 12 x 8
+// (2 times) where the larger one leaves SMs without work, with two threads per cell so
+// that a phase over the box is one pass: a stage of a short mesh lasts as long as one
+// CTA's chain of phases. Porous medium FP64, one stage at 32 x 8 / 12 x 8 with 96 threads
+// / with 192: 40^2 26.8 / 20.6 / 16.5 us, 100^2 31.8 / 25.6 / 20.5 us, 200^2 40.3 / 30.8 /
+// 28.2 us, 300^2 53.4 / 53.9 / 59.5 us, 600^2 155 / 167 / 186 us (8 x 8 and 8 x 4 tiles
+// were no faster on the short ones).
+template <int FLUX, class T, bool BLEND, bool RECT>
+static cudaError_t stage2d_go(const DevModel& m, const StageArgs2D<T>& a, cudaStream_t s) {
+  if constexpr (std::is_same_v<T, float> && !RECT) {
+    return launch_stream2d_f32(FLUX, BLEND ? (a.blend_external ? 2 : 1) : 0, m, a, s);
+  } else {
+    constexpr int H = BLEND ? 3 : 2;
+    if (tile_cost(a.nx, a.ny, 12, 8, H) < tile_cost(a.nx, a.ny, 32, 8, H))
+      return stage2d_tiles<FLUX, T, BLEND, RECT, 12, 8, 192>(m, a, s);
+    return stage2d_tiles<FLUX, T, BLEND, RECT, 32, 8>(m, a, s);
+  }
 }
 
 template <class T, bool RECT>

@@ -19,6 +19,7 @@
 // 5-point line is the fine points p - 2e .. p + 2e and a Simpson average weighs 1, 4, 1
 // per axis. Inputs are read from global memory (reuse through L1 / L2).
 #include "launch.h"
+#include "march3d_plan.h"
 #include "stage3d.cuh"
 
 namespace af {
@@ -484,9 +485,10 @@ cudaError_t dispatch3d(int flux, const DevModel& m, const StageArgs3D<T>& a, cud
 
 }  // namespace
 
-// without the blend one marching launch per output (march3d.cuh); with it the four kernels
+// without the blend one marching launch per output where that is faster (march3d_takes), else
+// the four kernels
 cudaError_t launch_stage3d_f64(int flux, const DevModel& m, const StageArgs3D<double>& a, cudaStream_t s) {
-  if (!a.blend) return launch_march3d_f64(flux, m, a, s);
+  if (!a.blend && march3d_takes(flux, true, a.n)) return launch_march3d_f64(m, a, s);
   return dispatch3d<double>(flux, m, a, s);
 }
 cudaError_t launch_stage3d_f32(int flux, const DevModel& m, const StageArgs3D<float>& a, cudaStream_t s) {

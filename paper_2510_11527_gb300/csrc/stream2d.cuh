@@ -653,7 +653,8 @@ __device__ __forceinline__ void blend_s_tile(const double* __restrict__ ub, int 
 // ---- launch (host)
 
 // Strip height of the column-marching kernel, at least 16 rows (the warm-up of a strip
-// is 4 rows). At 16 resident warps per SM (4 CTAs): about two and a half waves, at most
+// is 4 rows) where that gives every scheduler of the 152 SMs a warp; on smaller meshes, whose
+// stage lasts as long as one warp's march, shorter strips, down to 4 rows. At 16 resident warps per SM (4 CTAs): about two and a half waves, at most
 // 128 rows (measured stage times, degenerate Burgers: 1024^2 S = 8/12/16:
 // 0.0549/0.0544/0.0543 ms; 2048^2 S = 16/24/32/48: 0.1487/0.1451/0.1468/0.1494 ms;
 // 4096^2 S = 62/96/128: 0.477/0.471/0.508 ms). The heavier kernels at 12 warps per SM
@@ -664,7 +665,8 @@ static int stream_strip(int nx, int ny, bool heavy) {
   const long long bands = (nx + STREAM_BAND - 1) / STREAM_BAND;
   const long long target = heavy ? 152LL * 16 * 4 : 152LL * 16 * 5 / 2;
   long long S = (bands * ny + target - 1) / target;
-  if (S < 16) S = 16;
+  const long long fill = (bands * ny + 152 * 4 - 1) / (152 * 4);   // one warp per scheduler
+  if (S < 16) S = fill >= 16 ? 16 : (fill < 4 ? 4 : fill);
   if (S > (heavy ? 64 : 128)) S = heavy ? 64 : 128;
   return (int)S;
 }
