@@ -4,6 +4,7 @@
 // and the limiter function Theta (Section 5.1.1).
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "af.h"
@@ -28,6 +29,11 @@ struct DevModel {
   // the same parameters rounded to float, read by the FP32 stencils (GB300's FP64
   // unit also performs the double->float conversions, so none happen per use)
   float fpf[4], dpf[4], critf[2][8], critvf[2][8];
+  // FP32, limiter on: the extrema inside the bounds and their |f_l'| in two fixed slots per
+  // direction (an empty slot lies at infinity, inside no interval); crit_few = 0 when a
+  // direction has more of them or the state may leave the bounds
+  float critf2[2][2], critvf2[2][2];
+  int crit_few;
   int pme_e;             // AF_DIFF_PME: the integer exponent p0 (no conversion per use)
   // parts of the convex decomposition of each limited directional state u^{Lim,+-}
   // (Section 5.1.1, per direction in Section 5.2): 3 -- the face correction and the two
@@ -55,6 +61,30 @@ inline void fill_float_params(DevModel& m) {
     }
 }
 
+// after the bounds are known: DevModel::critf2 (a limited state stays inside the bounds up
+// to the safeguard's tolerance, so an extremum outside them by more is inside no interval
+// of two of its values). 2D only: a 1D end value may lie outside.
+inline void fill_few_criticals(DevModel& m, bool limiter, int dim) {
+  m.crit_few = limiter && dim == 2 ? 1 : 0;
+  const double margin = 1e-5 * (fabs(m.umin) > fabs(m.umax) ? fabs(m.umin) : fabs(m.umax));
+  for (int d = 0; d < 2; ++d) {
+    int n = 0;
+    for (int k = 0; k < 2; ++k) {
+      m.critf2[d][k] = INFINITY;
+      m.critvf2[d][k] = 0.0f;
+    }
+    for (int k = 0; k < m.ncrit[d]; ++k) {
+      if (m.crit[d][k] <= m.umin - margin || m.crit[d][k] >= m.umax + margin) continue;
+      if (n == 2) {
+        m.crit_few = 0;
+        break;
+      }
+      m.critf2[d][n] = m.critf[d][k];
+      m.critvf2[d][n++] = m.critvf[d][k];
+    }
+  }
+}
+
 // Comparisons, min and max of doubles run on the integer units through an
 // order-preserving 64-bit key (key(a) < key(b) <=> a < b for non-NaN values; -0 orders
 // just below +0): GB300's FP64 unit, which would otherwise execute DSETP/DMNMX, is the
@@ -77,22 +107,21 @@ __device__ __forceinline__ double tabs(double a) {
 }
 __device__ __forceinline__ float tabs(float a) { return fabsf(a); }
 
-// exact float -> double with integer operations only (finite inputs). A subnormal
-// float m * 2^-149 with leading bit p of m becomes the normal double
-// 1.f * 2^(p - 149); the FP64 unit is never used.
+// exact float -> double with integer operations only (finite inputs): the exponent is
+// rebiased by 896 in the high word; a zero keeps its word. A subnormal float m * 2^-149
+// with leading bit p of m becomes the normal double 1.f * 2^(p - 149). The FP64 unit is
+// never used.
 __device__ __forceinline__ double f2d_exact(float f) {
-  const unsigned int u = (unsigned int)__float_as_int(f);
-  const unsigned int e = (u >> 23) & 0xFFu;
-  const unsigned int mant = u & 0x7FFFFFu;
-  const unsigned long long s = (unsigned long long)(u & 0x80000000u) << 32;
-  if (e == 0u) {
-    if (mant == 0u) return __longlong_as_double((long long)s);
+  const unsigned int u = (unsigned int)__float_as_int(f), mag = u & 0x7FFFFFFFu;
+  if (mag - 1u < 0x007FFFFFu) {   // subnormal
+    const unsigned int mant = mag;
     const int p = 31 - __clz((int)mant);
+    const unsigned long long s = (unsigned long long)(u & 0x80000000u) << 32;
     const unsigned long long fr = ((unsigned long long)mant << (52 - p)) & 0xFFFFFFFFFFFFFull;
     return __longlong_as_double((long long)(s | ((unsigned long long)(p + 874) << 52) | fr));
   }
-  const unsigned long long d = s | ((unsigned long long)(e - 127u + 1023u) << 52) | ((unsigned long long)mant << 29);
-  return __longlong_as_double((long long)d);
+  const unsigned int hi = mag == 0u ? u : (u & 0x80000000u) | ((mag >> 3) + 0x38000000u);
+  return __hiloint2double((int)hi, (int)(u << 29));
 }
 
 // x == 0.0 (either sign) tested on the integer units
@@ -237,6 +266,16 @@ __device__ __forceinline__ T alpha_interval_pre(const DevModel& m, int dir, T a,
   } else if constexpr (FLUX == FLUX_BL) {
     const T lo = tmin(a, b), hi = tmax(a, b);
     T best = tmax(da, db);
+    if constexpr (sizeof(T) == 4) {
+      // the usual case without a loop (two compares and a select per slot): the loop, with
+      // its indexed constants, took most of a Buckley-Leverett LLF flux's instructions
+      if (m.crit_few) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+          if ((lo < m.critf2[dir][k]) & (m.critf2[dir][k] < hi)) best = tmax(best, m.critvf2[dir][k]);
+        return best;
+      }
+    }
     for (int k = 0; k < m.ncrit[dir]; ++k) {
       const T c = par<T>(m.crit[dir], m.critf[dir], k);
       if (tlt(lo, c) && tlt(c, hi)) best = tmax(best, par<T>(m.critv[dir], m.critvf[dir], k));

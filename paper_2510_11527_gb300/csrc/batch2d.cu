@@ -18,6 +18,7 @@
 #include "model_host.h"
 #include "reduce.cuh"
 #include "batch2d.cuh"
+#include "strip_plan.h"
 
 namespace af {
 
@@ -332,22 +333,17 @@ af_status build_work(af_batch* b) {
     for (int t = 0; t < I.tiles_x * tiles_y; ++t) work.push_back(k);
   }
   b->total_tiles = (int)work.size();
-  // column-marching items of every instance (FP32-mixed without the blend). Strip
-  // height: the tallest of 128, 64, 32 rows that still gives every resident warp slot
-  // (SMs x resident warps) at least 8 items -- each strip repeats a 4-row warm-up and its
-  // setup, so taller strips cost less per row (256 instances of 64^2..1024^2: S = 32
-  // 1.57e10, 64 1.77e10, 128 1.86e10 cell-stage/s)
+  // column-marching items of every instance (FP32-mixed); the strip height as on a single
+  // mesh (12 resident warps per SM for Buckley-Leverett and the blend, else 16)
   {
-    long long rows = 0;
-    for (int k = 0; k < b->n; ++k)
-      rows += (long long)((b->h_inst[k].nx + af::BATCH_STREAM_BAND - 1) / af::BATCH_STREAM_BAND) * b->h_inst[k].ny;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
-    // resident warps per SM of the column-marching kernel: 12 for Buckley-Leverett and
-    // the blend (3 CTAs of 4 warps), else 16
-    const long long want = 8LL * ((b->blend || b->flux == AF_FLUX_BL) ? 12 : 16) * sms;
-    b->stream_S = rows / 128 >= want ? 128 : (rows / 64 >= want ? 64 : 32);
+    const bool heavy = b->blend || b->flux == AF_FLUX_BL;
+    b->stream_S = af::strip_plan(heavy ? af::MARCH_HEAVY : af::MARCH_LIGHT, [&](int S) {
+      long long n = 0;
+      for (int k = 0; k < b->n; ++k)
+        n += (long long)((b->h_inst[k].nx + af::BATCH_STREAM_BAND - 1) / af::BATCH_STREAM_BAND) *
+             ((b->h_inst[k].ny + S - 1) / S);
+      return n;
+    }).S;
   }
   std::vector<int> items;
   for (int k = 0; k < b->n; ++k) {
@@ -485,6 +481,7 @@ af_status af_batch_create(int n, const af_grid* grids, const af_flux* fluxes, co
     I.m.umin = bounds[k].umin;
     I.m.umax = bounds[k].umax;
     af::finish_model(I.m, fluxes[k].kind, 2);
+    af::fill_few_criticals(I.m, opts->limiter != 0, 2);
     I.kmax = af::kappa_max_of(diffs[k], bounds[k].umin, bounds[k].umax);
     const double scale = std::max(std::fabs(bounds[k].umin), std::fabs(bounds[k].umax));
     I.tol = (b->prec == AF_PREC_FP64 ? 8.0 * 2.220446049250313e-16 : 64.0 * 1.1920929e-07) * scale;

@@ -467,6 +467,7 @@ af_status af_create(const af_grid* grid, const af_flux* flux, const af_diff* dif
   c->m.umin = bounds->umin;
   c->m.umax = bounds->umax;
   af::finish_model(c->m, flux->kind, grid->dim);
+  if (!c->bounds_pending) af::fill_few_criticals(c->m, opts->limiter != 0, grid->dim);
   if (!c->bounds_pending) c->kmax = af::kappa_max_of(*diff, bounds->umin, bounds->umax);
   const double scale = std::max(std::fabs(bounds->umin), std::fabs(bounds->umax));
   c->tol = (c->prec == AF_PREC_FP64 ? 8.0 * 2.220446049250313e-16 : 64.0 * 1.1920929e-07) * scale;
@@ -571,6 +572,7 @@ af_status af_set_state(af_ctx* c, const double* ub, const double* V, const doubl
     c->m.umin = lo;
     c->m.umax = hi;
     c->m.umid = 0.5 * (lo + hi);
+    af::fill_few_criticals(c->m, c->opts.limiter != 0, c->dim);
     c->kmax = af::kappa_max_of(c->diff, lo, hi);
     const double scale = std::max(std::fabs(lo), std::fabs(hi));
     c->tol = (c->prec == AF_PREC_FP64 ? 8.0 * 2.220446049250313e-16 : 64.0 * 1.1920929e-07) * scale;
@@ -670,6 +672,7 @@ af_status af_set_state_arrays(af_ctx* c, int narr, const double* const* arrays) 
     c->m.umin = lo;
     c->m.umax = hi;
     c->m.umid = 0.5 * (lo + hi);
+    af::fill_few_criticals(c->m, c->opts.limiter != 0, c->dim);
     c->kmax = af::kappa_max_of(c->diff, lo, hi);
     c->tol = (c->prec == AF_PREC_FP64 ? 8.0 * 2.220446049250313e-16 : 64.0 * 1.1920929e-07) *
              std::max(std::fabs(lo), std::fabs(hi));

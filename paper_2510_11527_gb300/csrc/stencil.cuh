@@ -13,6 +13,19 @@ __device__ __forceinline__ float fmn(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ double fmx(double a, double b) { return tmax(a, b); }
 __device__ __forceinline__ double fmn(double a, double b) { return tmin(a, b); }
 
+// largest / smallest of three (one instruction in FP32) and of five
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max5(float a, float b, float c, float d, float e) { return max3(max3(a, b, c), d, e); }
+
 // Diffusion kinds compiled into the column-marching kernel (DK_GENERIC takes the
 // model's runtime kind).
 enum : int { DK_GENERIC = -1, DK_NONE = 0, DK_CONST = 1, DK_PWL = 2, DK_PME2 = 3, DK_CUBIC = 4 };

@@ -22,6 +22,7 @@
 #pragma once
 #include "stage2d.cuh"
 #include "stencil.cuh"
+#include "strip_plan.h"
 
 namespace af {
 
@@ -95,9 +96,9 @@ template <int FLUX, class T>
 __device__ __forceinline__ T line_alpha(const DevModel& m, int dir, T z0, T z1, T z2, T z3, T z4, T d0, T d1, T d2,
                                         T d3, T d4) {
   if constexpr (FLUX == FLUX_BURGERS) {
-    return tabs(T(2) * par<T>(m.fp, m.fpf, 0)) * fmx(fmx(fmx(tabs(z0), tabs(z1)), fmx(tabs(z3), tabs(z4))), tabs(z2));
+    return tabs(T(2) * par<T>(m.fp, m.fpf, 0)) * max5(tabs(z0), tabs(z1), tabs(z2), tabs(z3), tabs(z4));
   } else if constexpr (FLUX == FLUX_BL) {
-    return fmx(fmx(fmx(d0, d1), fmx(d3, d4)), d2);
+    return max5(d0, d1, d2, d3, d4);
   } else if constexpr (FLUX == FLUX_LINEAR) {
     return tabs(T(dir == 0 ? m.fp[0] : m.fp[1]));
   } else {
@@ -348,10 +349,12 @@ __device__ __forceinline__ void stream_step(const StreamCtx<FLUX, DIFF, T>& c, i
                 cur.ULm2 + e2};
     T lo = zh[0], hi = zh[0];
 #pragma unroll
-    for (int q = 1; q < 12; ++q) {
-      lo = fmn(lo, zh[q]);
-      hi = fmx(hi, zh[q]);
+    for (int q = 1; q < 11; q += 2) {
+      lo = min3(lo, zh[q], zh[q + 1]);
+      hi = max3(hi, zh[q], zh[q + 1]);
     }
+    lo = fmn(lo, zh[11]);
+    hi = fmx(hi, zh[11]);
     if (tlt(lo, k.umin) | tlt(k.umax, hi)) {
       T t[12];
 #pragma unroll
@@ -409,7 +412,7 @@ __device__ __forceinline__ void stream_step(const StreamCtx<FLUX, DIFF, T>& c, i
     }
     // post-stage safeguard: one test for the four values, the clamp path only if needed
     if (lim && A.sg[0] &&
-        (tlt(ubo, m.umin) | tlt(m.umax, ubo) | (fmn(fmn(vo, xo), yo) < k.umin) | (fmx(fmx(vo, xo), yo) > k.umax))) {
+        (tlt(ubo, m.umin) | tlt(m.umax, ubo) | (min3(vo, xo, yo) < k.umin) | (max3(vo, xo, yo) > k.umax))) {
       ubo = safeguard<double>(ubo, m.umin, m.umax, A.tol, A.stats, true);
       vo = safeguard<T>(vo, k.umin, k.umax, A.tol, A.stats);
       xo = safeguard<T>(xo, k.umin, k.umax, A.tol, A.stats);
@@ -652,49 +655,42 @@ __device__ __forceinline__ void blend_s_tile(const double* __restrict__ ub, int 
 
 // ---- launch (host)
 
-// Strip height of the column-marching kernel, at least 16 rows (the warm-up of a strip
-// is 4 rows) where that gives every scheduler of the 152 SMs a warp; on smaller meshes, whose
-// stage lasts as long as one warp's march, shorter strips, down to 4 rows. At 16 resident warps per SM (4 CTAs): about two and a half waves, at most
-// 128 rows (measured stage times, degenerate Burgers: 1024^2 S = 8/12/16:
-// 0.0549/0.0544/0.0543 ms; 2048^2 S = 16/24/32/48: 0.1487/0.1451/0.1468/0.1494 ms;
-// 4096^2 S = 62/96/128: 0.477/0.471/0.508 ms). The heavier kernels at 12 warps per SM
-// (Buckley-Leverett, the blend) keep about four waves of 16 warps and at most 64 rows:
-// the blended Buckley-Leverett stage at 4096^2 lost 4 % at S = 100 (3.3 waves, the last
-// one partly filled) against S = 62.
-static int stream_strip(int nx, int ny, bool heavy) {
-  const long long bands = (nx + STREAM_BAND - 1) / STREAM_BAND;
-  const long long target = heavy ? 152LL * 16 * 4 : 152LL * 16 * 5 / 2;
-  long long S = (bands * ny + target - 1) / target;
-  const long long fill = (bands * ny + 152 * 4 - 1) / (152 * 4);   // one warp per scheduler
-  if (S < 16) S = fill >= 16 ? 16 : (fill < 4 ? 4 : fill);
-  if (S > (heavy ? 64 : 128)) S = heavy ? 64 : 128;
-  return (int)S;
+// the strip height of a single mesh (strip_plan.h)
+static StripPlan stream_plan(int nx, int ny, bool heavy, bool zero) {
+  const int bands = (nx + STREAM_BAND - 1) / STREAM_BAND;
+  return strip_plan(heavy ? MARCH_HEAVY : (zero ? MARCH_ZERO : MARCH_LIGHT),
+                    [=](int S) { return (long long)bands * ((ny + S - 1) / S); });
+}
+
+// the stage arguments of output o alone
+static StageArgs2D<float> one_output(const StageArgs2D<float>& a, int o) {
+  StageArgs2D<float> b = a;
+  b.nout = 1;
+  b.tcoef[0] = a.tcoef[o];
+  b.cA[0] = a.cA[o];
+  b.cF[0] = a.cF[o];
+  b.Aub[0] = a.Aub[o];
+  b.AV[0] = a.AV[o];
+  b.AX[0] = a.AX[o];
+  b.AY[0] = a.AY[o];
+  b.Oub[0] = a.Oub[o];
+  b.OV[0] = a.OV[o];
+  b.OX[0] = a.OX[o];
+  b.OY[0] = a.OY[o];
+  b.sg[0] = a.sg[o];
+  return b;
 }
 
 // one launch per output of the stage
 template <int FLUX, int DIFF, int BK = 0>
 static cudaError_t stream2d_go(const DevModel& m, const StageArgs2D<float>& a, cudaStream_t s) {
-  const int S = stream_strip(a.nx, a.ny, stream_min_blocks<FLUX, BK>() < 4);
+  const int S = stream_plan(a.nx, a.ny, stream_min_blocks<FLUX, BK>() < 4, FLUX == FLUX_ZERO).S;
   const int bands = (a.nx + STREAM_BAND - 1) / STREAM_BAND;
   const long long warps = (long long)bands * ((a.ny + S - 1) / S);
   const long long blocks = (warps + STREAM_WPB - 1) / STREAM_WPB;
   if (blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
   for (int o = 0; o < a.nout; ++o) {
-    StageArgs2D<float> b = a;
-    b.nout = 1;
-    b.tcoef[0] = a.tcoef[o];
-    b.cA[0] = a.cA[o];
-    b.cF[0] = a.cF[o];
-    b.Aub[0] = a.Aub[o];
-    b.AV[0] = a.AV[o];
-    b.AX[0] = a.AX[o];
-    b.AY[0] = a.AY[o];
-    b.Oub[0] = a.Oub[o];
-    b.OV[0] = a.OV[o];
-    b.OX[0] = a.OX[o];
-    b.OY[0] = a.OY[o];
-    b.sg[0] = a.sg[o];
-    stream2d_kernel<FLUX, DIFF, BK><<<(unsigned)blocks, 32 * STREAM_WPB, 0, s>>>(m, b, S, bands);
+    stream2d_kernel<FLUX, DIFF, BK><<<(unsigned)blocks, 32 * STREAM_WPB, 0, s>>>(m, one_output(a, o), S, bands);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
