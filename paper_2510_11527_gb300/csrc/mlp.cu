@@ -393,6 +393,11 @@ __device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
   return z ^ (z >> 31);
 }
 
+// programmatic dependent launch (sm_90 and later): let the next launch of the stream start,
+// and wait for the completion of the one before
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Forward + backward of a minibatch in FP32 with the tensor-core path's rounding points
 // (bf16 inputs and weights of the two hidden layers): the gradient of the batch-mean loss
 // summed over the samples of each CTA into its row of `partial` (TRAIN_ROW floats: the
@@ -408,6 +413,12 @@ __device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
 // warp's chain is an eighth of the network's. The weight gradients are products of two
 // [unit][sample] arrays in shared memory, 4 + 3 entries per thread, kept in registers over
 // the CTA's tiles. Sums over a layer's inputs run in the order of the single-sample form.
+//
+// A step is two short dependent launches (this one and adam_kernel), each launched while
+// the one before still runs (programmatic dependent launch): the loads that do not depend
+// on it -- the first tile's sample indices, features and targets -- are made before
+// griddepcontrol.wait, which returns when the launch before has completed and its writes
+// are visible.
 constexpr int TRAIN_TILE = 32;            // samples per tile (one per lane)
 constexpr int TRAIN_LD = TRAIN_TILE + 4;  // row stride: 16-byte aligned, 8 rows on distinct banks
 constexpr int TRAIN_MAX_CTAS = 152 * 2;   // rows of the partial sums
@@ -421,6 +432,29 @@ __global__ void __launch_bounds__(256, 2) train_kernel(const float* __restrict__
   __shared__ __align__(16) float xT[NIN][TRAIN_LD], h1T[NH][TRAIN_LD], h2T[NH][TRAIN_LD];
   __shared__ __align__(16) float d1T[NH][TRAIN_LD], d2T[NH][TRAIN_LD], d3[TRAIN_LD];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  launch_dependents();
+  const int tiles = (batch - 1) / TRAIN_TILE + 1;
+  // a tile's targets (one per lane) and this warp's four sample rows (one input per lane)
+  float target = 0.f, rows[4];
+  bool live = false;
+  auto fetch = [&](int tile) {
+    const long long k = (long long)tile * TRAIN_TILE + lane;
+    live = k < batch;
+    long long idx = 0;
+    if (live)
+      idx = seed == 0 ? k
+                      : (long long)(splitmix64(seed ^ ((unsigned long long)step << 32) ^ (unsigned long long)k) %
+                                    (unsigned long long)nsamples);
+    target = live ? label[idx] : 0.f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int sl = 4 * warp + r;
+      const long long row = __shfl_sync(0xffffffffu, idx, sl);
+      rows[r] = lane < NIN && k - lane + sl < batch ? bfr(feat[row * NIN + lane]) : 0.f;
+    }
+  };
+  if (blockIdx.x < tiles) fetch(blockIdx.x);
+  grid_dependency_wait();
   for (int k = tid; k < NH * NIN; k += 256) W1T[k % NIN][k / NIN] = bfr(params[OFF_W1 + k]);
   for (int k = tid; k < NH * NH; k += 256) {
     const float w = bfr(params[OFF_W2 + k]);
@@ -437,23 +471,12 @@ __global__ void __launch_bounds__(256, 2) train_kernel(const float* __restrict__
   // gq + 8 k < 21) and one entry of b1, b2, w3 or b3
   const int go = tid >> 3, gq = tid & 7;
   float gw2[4] = {0.f, 0.f, 0.f, 0.f}, gw1[3] = {0.f, 0.f, 0.f}, gb = 0.f, lossv = 0.f;
-  const int tiles = (batch - 1) / TRAIN_TILE + 1;
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const long long k = (long long)tile * TRAIN_TILE + lane;
-    const bool live = k < batch;
-    long long idx = 0;
-    if (live)
-      idx = seed == 0 ? k
-                      : (long long)(splitmix64(seed ^ ((unsigned long long)step << 32) ^ (unsigned long long)k) %
-                                    (unsigned long long)nsamples);
-    const float target = live ? label[idx] : 0.f;
+    if (tile != (int)blockIdx.x) fetch(tile);
     __syncthreads();   // the previous tile's arrays have been read (and the weights written)
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {   // rows 4 warp .. 4 warp + 3, one coalesced read each
-      const int sl = 4 * warp + r;
-      const long long row = __shfl_sync(0xffffffffu, idx, sl);
-      if (lane < NIN) xT[lane][sl] = k - lane + sl < batch ? bfr(feat[row * NIN + lane]) : 0.f;
-    }
+    for (int r = 0; r < 4; ++r)
+      if (lane < NIN) xT[lane][4 * warp + r] = rows[r];
     __syncthreads();
     const int u0 = 4 * warp;   // this warp's units of each layer
     float z1[4] = {0.f, 0.f, 0.f, 0.f};
@@ -572,7 +595,7 @@ __device__ __forceinline__ float column_sum(const float* __restrict__ partial, i
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = blockIdx.x * 32 + lane;
   float acc = 0.f;
   if (q <= NPARAM) {
-#pragma unroll 4
+#pragma unroll 16
     for (int r = warp; r < rows; r += 8) acc += partial[(size_t)r * TRAIN_ROW + q];
   }
   sm[warp][lane] = acc;
@@ -589,6 +612,8 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ p, float*
                                                    float* __restrict__ v, const float* __restrict__ partial, int rows,
                                                    float lr, float c1, float c2, __nv_bfloat16* w1q,
                                                    __nv_bfloat16* w2q, float* __restrict__ loss) {
+  launch_dependents();
+  grid_dependency_wait();
   const float g = column_sum(partial, rows);
   const int q = blockIdx.x * 32 + (int)threadIdx.x;
   if (threadIdx.x >= 32 || q > NPARAM) return;
@@ -667,6 +692,20 @@ cudaError_t mlp_indicator_batch_launch(const af_mlp* net, const BatchInst* inst,
 }  // namespace af
 
 namespace {
+// launch that may start while the launch before it in the stream runs (its kernel waits)
+template <class... P, class... A>
+cudaError_t launch_early(void (*kern)(P...), int grid, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(256);
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // CTAs (rows of partial sums) of a minibatch
 int train_rows(int batch) { return std::min((batch - 1) / TRAIN_TILE + 1, TRAIN_MAX_CTAS); }
 }  // namespace
@@ -773,11 +812,17 @@ af_status af_mlp_train(af_mlp* net, const float* feat_dev, const float* label_de
   float last = 0.f;
   const int rows = train_rows(batch);
   for (int s = 0; s < steps; ++s) {
-    train_kernel<<<rows, 256>>>(feat_dev, label_dev, nsamples, batch, seed, s, net->params, net->partial);
+    // (the first launch waits for the stream as usual: the rows may just have been written)
+    if (s == 0)
+      train_kernel<<<rows, 256>>>(feat_dev, label_dev, nsamples, batch, seed, s, net->params, net->partial);
+    else if (launch_early(train_kernel, rows, feat_dev, label_dev, nsamples, batch, seed, s, net->params,
+                          net->partial) != cudaSuccess)
+      return AF_E_CUDA;
     net->t += 1;
     const float c1 = 1.f - powf(0.9f, (float)net->t), c2 = 1.f - powf(0.999f, (float)net->t);
-    adam_kernel<<<COLUMN_CTAS, 256>>>(net->params, net->m, net->v, net->partial, rows, lr, c1, c2, net->w1q, net->w2q,
-                                      net->loss);
+    if (launch_early(adam_kernel, COLUMN_CTAS, net->params, net->m, net->v, net->partial, rows, lr, c1, c2, net->w1q,
+                     net->w2q, net->loss) != cudaSuccess)
+      return AF_E_CUDA;
     if (cudaGetLastError() != cudaSuccess) return AF_E_CUDA;
     if (s == steps - 1 && loss_host) {
       if (cudaMemcpy(&last, net->loss, sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess) return AF_E_CUDA;

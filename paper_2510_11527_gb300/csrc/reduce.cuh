@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
                                                                const double* __restrict__ ub,
                                                                unsigned long long* rate_bits, int bc, double gl,
                                                                double gr, const DtFinal fin) {
-  const size_t n = (size_t)nx * ny;
+  static_assert(FLUX == FLUX_BL, "the other fluxes take dt_rate_maxu_kernel");
   double best = 0.0;
   unsigned flags = 0u;
   const double kd1 = kmax * inv_h1 * inv_h1, kd2 = kmax * inv_h2 * inv_h2;
@@ -154,6 +154,8 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
   // ulps). The FP64 one costs a division on GB300's slow FP64 unit, so it is formed only
   // for the cells whose estimate is within 2^-12 of the block's largest estimate: the
   // cell with the largest FP64 rate is always among them, so the maximum is the same.
+  // (Finding each cell's coordinates by 64-bit divisions, and estimating every cell twice,
+  // had cost most of the kernel: 0.28 ms per step at 4096^2.)
   auto rate64 = [&](double u) {
     const BLVals<double> r = bl_eval<double>(m, u);
     double b = r.d[dim == 1 ? 1 : 0] * inv_h1 + kd1;
@@ -167,59 +169,66 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
     if (dim == 2) b = fmaxf(b, r.d[1] * ih2f + kd2f);
     return b;
   };
+  // cells in segments of up to RATE_SEG columns of a row, so that a thread's cells need no
+  // division to find their coordinates
+  constexpr int RATE_SEG = 4 * RED_THREADS;
+  const int spr = (nx + RATE_SEG - 1) / RATE_SEG;   // segments per row
+  const long long nseg = (long long)spr * ny;
+  auto cells = [&](auto&& f) {
+    for (long long sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
+      const int j = (int)(sg / spr), b = (int)(sg - (long long)j * spr) * RATE_SEG;
+      if (rect && j == 0) continue;
+      const int e = min(b + RATE_SEG, nx);
+      for (int i = b + (int)threadIdx.x; i < e; i += RED_THREADS)
+        if (!(rect && i == 0)) f(i, j, (size_t)j * nx + i);
+    }
+  };
+  auto bits_of = [](double u) { return (unsigned long long)__double_as_longlong(u); };
   float m32 = 0.0f;
-  for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(k % nx), j = (int)(k / nx);
-    if (rect && (i == 0 || j == 0)) continue;
-    const double u = ub[k];
-    if constexpr (FLUX == FLUX_BL) {
-      m32 = fmaxf(m32, rate32(u));
+  {
+    unsigned long long last = ~0ull;   // bits of the last u evaluated (NaN: none)
+    cells([&](int i, int j, size_t k) {
+      const double u = ub[k];
+      if (bits_of(u) != last) {
+        m32 = fmaxf(m32, rate32(u));
+        last = bits_of(u);
+      }
+      // an extremum lies strictly inside a face's interval only if its ends differ
       double un = ub[(size_t)j * nx + (i + 1 == nx ? 0 : i + 1)];
       if (dim == 1 && bc != AF_BC_PERIODIC && i + 1 == nx) un = bc == AF_BC_DIRICHLET ? gr : u;
       if (rect && i + 1 == nx) un = u;
-      flags |= crit_flags<FLUX>(m, 0, u, un);
+      if (bits_of(un) != bits_of(u)) flags |= crit_flags<FLUX>(m, 0, u, un);
       if (dim == 1 && bc == AF_BC_DIRICHLET && k == 0) flags |= crit_flags<FLUX>(m, 0, gl, u);
       if (dim == 2) {
         const double ut = (rect && j + 1 == ny) ? u : ub[(size_t)(j + 1 == ny ? 0 : j + 1) * nx + i];
-        flags |= crit_flags<FLUX>(m, 1, u, ut) << 8;
+        if (bits_of(ut) != bits_of(u)) flags |= crit_flags<FLUX>(m, 1, u, ut) << 8;
       }
-    } else {
-      best = tmax(best, alpha_interval<FLUX, double>(m, 0, u, u) * inv_h1 + kd1);
-      if (dim == 2) best = tmax(best, alpha_interval<FLUX, double>(m, 1, u, u) * inv_h2 + kd2);
-    }
+    });
   }
-  if constexpr (FLUX == FLUX_BL) {
+  {
+    const float mine = m32;   // the largest estimate among this thread's cells
     __shared__ float s32[RED_THREADS / 32];
     for (int o = 16; o > 0; o >>= 1) m32 = fmaxf(m32, __shfl_xor_sync(0xffffffffu, m32, o));
     if ((threadIdx.x & 31) == 0) s32[threadIdx.x >> 5] = m32;
     __syncthreads();
     for (int w = 0; w < RED_THREADS / 32; ++w) m32 = fmaxf(m32, s32[w]);
     const float thr = m32 - m32 * (1.0f / 4096.0f);
-    unsigned long long last = ~0ull;   // bits of the last u evaluated in FP64 (NaN: none)
-    double lastr = 0.0;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-      if (rect) {
-        const int i = (int)(k % nx), j = (int)(k / nx);
-        if (i == 0 || j == 0) continue;
-      }
-      const double u = ub[k];
-      if (rate32(u) < thr) continue;
-      const unsigned long long bits = (unsigned long long)__double_as_longlong(u);
-      if (bits != last) {
+    if (mine >= thr) {   // only threads with a candidate look at their cells again
+      unsigned long long last = ~0ull;
+      double lastr = 0.0;
+      cells([&](int, int, size_t k) {
+        const double u = ub[k];
+        if (bits_of(u) == last) return;
+        if (rate32(u) < thr) return;
         lastr = rate64(u);
-        last = bits;
-      }
-      best = tmax(best, lastr);
+        last = bits_of(u);
+        best = tmax(best, lastr);
+      });
     }
   }
   if (dim == 1 && bc == AF_BC_DIRICHLET && blockIdx.x == 0 && threadIdx.x == 0) {
     const double gv[2] = {gl, gr};
-    for (int s = 0; s < 2; ++s) {
-      double d;
-      if constexpr (FLUX == FLUX_BL) d = bl_eval<double>(m, gv[s]).d[1];
-      else d = alpha_interval<FLUX, double>(m, 0, gv[s], gv[s]);
-      best = tmax(best, d * inv_h1 + kd1);
-    }
+    for (int s = 0; s < 2; ++s) best = tmax(best, bl_eval<double>(m, gv[s]).d[1] * inv_h1 + kd1);
   }
   for (int o = 16; o > 0; o >>= 1) best = tmax(best, __shfl_xor_sync(0xffffffffu, best, o));
   flags = __reduce_or_sync(0xffffffffu, flags);

@@ -652,7 +652,6 @@ __device__ __forceinline__ void blend_s_tile(const double* __restrict__ ub, int 
   }
 }
 
-
 // ---- launch (host)
 
 // the strip height of a single mesh (strip_plan.h)

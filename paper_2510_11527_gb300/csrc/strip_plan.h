@@ -2,14 +2,15 @@
 //
 // Every warp marches S rows plus about 5 steps of warm-up and setup; CTAs of 4 warps are
 // dealt to the SMs and R of them are resident. How long a step is depends on how many CTAs
-// share the SM: t[r - 1] microseconds with r of them. Two estimates of a launch are
-// averaged: its work at full residency, and its waves (the busiest SM's CTAs, R at a time),
-// because CTAs are equal on smooth data and uneven where the limiter works. To that comes
-// the tail, half of one strip's time on its own: fewer, taller strips repeat less warm-up
-// but one strip along a front then lasts past all others (degenerate Burgers 2048^2, per
-// step: 0.44 ms with 16 to 32 rows, 0.54 with 64 in one wave). Measured per stage against
-// the fixed number of waves used before, smooth data: Burgers 100^2 23 -> 11 us, 1200^2
-// 58 -> 45 us, Buckley-Leverett 1024^2 101 -> 54 us (with its loop-free wave speeds).
+// share the SM: t[r - 1] microseconds with r of them. A launch is estimated as its work at
+// full residency plus `tail` times one strip's time alone: taller strips repeat less
+// warm-up, but a strip along a front, where the limiter works, lasts past all others
+// (degenerate Burgers 2048^2, per step: 0.44 ms with 16 to 26 rows, 0.48 with 32, 0.56 with
+// 64 in one wave). The heavy kernels' strips are alike, so for them whole waves count (the
+// busiest SM's CTAs, R at a time) as much as the work (blended Buckley-Leverett 2048^2: 28
+// rows, 3.0 waves, 1.14 ms; 26 rows 1.26 ms). Measured per stage against the fixed number of
+// waves used before: Burgers 100^2 23 -> 12 us, 512^2 25 -> 17 us; Buckley-Leverett 1024^2
+// 101 -> 54 us (with its loop-free wave speeds).
 #pragma once
 
 namespace af {
@@ -22,22 +23,23 @@ struct StripPlan {
 struct MarchKind {
   int R;
   double t[4];
+  double waves, tail;   // weights of the waves (against the work) and of the tail
 };
-constexpr MarchKind MARCH_LIGHT = {4, {1.12, 1.25, 1.50, 1.72}};   // one column per lane
-constexpr MarchKind MARCH_ZERO = {4, {1.05, 1.18, 1.40, 1.60}};    // the same, zero flux
-constexpr MarchKind MARCH_HEAVY = {3, {0.68, 0.82, 1.00, 0.0}};    // Buckley-Leverett, blends (relative)
-constexpr MarchKind MARCH_PAIR = {3, {1.22, 1.40, 1.69, 0.0}};     // two columns per lane (zero flux)
+constexpr MarchKind MARCH_LIGHT = {4, {1.12, 1.25, 1.50, 1.72}, 0.0, 1.0};   // one column per lane
+constexpr MarchKind MARCH_ZERO = {4, {1.05, 1.18, 1.40, 1.60}, 0.0, 1.0};    // the same, zero flux
+constexpr MarchKind MARCH_HEAVY = {3, {0.68, 0.82, 1.00, 0.0}, 0.5, 0.7};    // Buckley-Leverett, blends (relative)
+constexpr MarchKind MARCH_PAIR = {3, {1.22, 1.40, 1.69, 0.0}, 0.0, 1.0};     // two columns per lane (zero flux)
 
 // warps(S): how many warps strips of S rows make
 template <class F>
 inline StripPlan strip_plan(const MarchKind& k, F&& warps) {
   StripPlan best{4, -1.0};
   for (int S = 4; S <= 128; S += S < 32 ? 1 : 4) {
-    const long long w = warps(S), q = (w + 4 * 152 - 1) / (4 * 152);   // q: CTAs of the busiest SM
+    const long long w = warps(S), q = (w + 4 * 152 * 97 / 100) / (4 * 152);   // CTAs of the busiest SM, but for a few
     const int rest = (int)(q % k.R);
     const double waves = (double)(q / k.R) * k.t[k.R - 1] + (rest ? k.t[rest - 1] : 0.0);
     const double work = (double)w / (4 * 152) * k.t[k.R - 1] / k.R;
-    const double cost = (S + 5) * (0.5 * (waves + work) + 0.5 * k.t[0]);
+    const double cost = (S + 5) * (k.waves * waves + (1.0 - k.waves) * work + k.tail * k.t[0]);
     if (best.cost < 0.0 || cost < best.cost) best = StripPlan{S, cost};
   }
   return best;
