@@ -62,8 +62,10 @@ inline void fill_float_params(DevModel& m) {
 }
 
 // after the bounds are known: DevModel::critf2 (a limited state stays inside the bounds up
-// to the safeguard's tolerance, so an extremum outside them by more is inside no interval
-// of two of its values). 2D only: a 1D end value may lie outside.
+// to the safeguard's tolerance -- data outside them are refused -- so an extremum outside
+// them by more is inside no interval of two of its values). 2D only: a 1D end value may
+// lie outside. (Three slots, enough for all extrema on the line without a look at the
+// bounds, cost 6 %: blended Buckley-Leverett step at 4096^2 3.94 / 4.19 ms.)
 inline void fill_few_criticals(DevModel& m, bool limiter, int dim) {
   m.crit_few = limiter && dim == 2 ? 1 : 0;
   const double margin = 1e-5 * (fabs(m.umin) > fabs(m.umax) ? fabs(m.umin) : fabs(m.umax));
