@@ -376,19 +376,24 @@ template <class T>
 __device__ __forceinline__ bool inb(T z, T umin, T umax) {
   return !tlt(z, umin) & !tlt(umax, z);
 }
-// min of Theta over two / four (zL, zH) pairs. In FP64 the common case (every zH inside
-// the bounds, so the minimum is 1) is tested first with integer compares; in FP32 the
-// plain evaluation measured as fast.
+// min of Theta over two / four (zL, zH) pairs. The common case (every zH inside the
+// bounds, so the minimum is 1) is tested first: in FP64 with integer compares, in FP32 by
+// the least and the largest zH (rectangle of Example 6.9, one FP32 step at 1536^2: 495 ->
+// 477 us; a NaN among them counts as inside in both forms).
 template <class T>
 __device__ __forceinline__ T theta_pair(T a0, T a1, T b0, T b1, T umin, T umax) {
   if constexpr (sizeof(T) == 8)
     if (inb(a1, umin, umax) & inb(b1, umin, umax)) return T(1);
+  if constexpr (sizeof(T) == 4)
+    if (tmin(a1, b1) >= umin && tmax(a1, b1) <= umax) return T(1);
   return tmin(theta_fn<T>(a0, a1, umin, umax), theta_fn<T>(b0, b1, umin, umax));
 }
 template <class T>
 __device__ __forceinline__ T theta_quad(T a0, T a1, T b0, T b1, T c0, T c1, T d0, T d1, T umin, T umax) {
   if constexpr (sizeof(T) == 8)
     if (inb(a1, umin, umax) & inb(b1, umin, umax) & inb(c1, umin, umax) & inb(d1, umin, umax)) return T(1);
+  if constexpr (sizeof(T) == 4)
+    if (tmin(tmin(a1, b1), tmin(c1, d1)) >= umin && tmax(tmax(a1, b1), tmax(c1, d1)) <= umax) return T(1);
   return tmin(tmin(theta_fn<T>(a0, a1, umin, umax), theta_fn<T>(b0, b1, umin, umax)),
               tmin(theta_fn<T>(c0, c1, umin, umax), theta_fn<T>(d0, d1, umin, umax)));
 }
