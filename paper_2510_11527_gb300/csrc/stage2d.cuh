@@ -369,7 +369,7 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
   const T umin = sc.umin, umax = sc.umax;
 
   // ---- P1: centres and pointwise nonlinearities ----------------------------------------
-  auto eval_point = [&](int type, int b) {
+  auto eval_point = [&](auto kc, int type, int b) {
     const T z = sZ[type][b];
     if constexpr (FLUX == FLUX_BURGERS) {
       Q(type, 0)[b] = flux<FLUX, T>(m, 0, z);
@@ -380,7 +380,7 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
       Q(type, PS::DOFF)[b] = r.d[0];
       Q(type, PS::DOFF + 1)[b] = r.d[1];
     }
-    Q(type, NQ - 1)[b] = apot<T>(m, z);
+    Q(type, NQ - 1)[b] = apot_as<decltype(kc)::value, T>(m, z);
   };
   T* sS1 = nullptr;
   T* sS2 = nullptr;
@@ -396,56 +396,59 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
     sTD1 = sS1;   // theta^{d,s} replaces s in place once theta^{c,s} is formed
     sTD2 = sS2;
   }
-  const auto p1_qu = seg<0, BX, 0, BY>([&](int bx, int by) {
-    const int k = by * BX + bx;
-    const T u = sU[k];
-    if constexpr (FLUX == FLUX_BURGERS) {
-      sQU[k] = flux<FLUX, T>(m, 0, u);
-    } else if constexpr (FLUX == FLUX_BL) {
-      const BLVals<T> r = bl_eval<T>(m, u);
-      sQU[k] = r.f[0];
-      if constexpr (PS::F2) sQU[BN + k] = r.f[1];
-      sQU[PS::DOFF * BN + k] = r.d[0];
-      sQU[(PS::DOFF + 1) * BN + k] = r.d[1];
-    }
-    sQU[(L::NQU - 1) * BN + k] = apot<T>(m, u);
-  });
-  const auto p1_pts = seg<H - 2, H + TX + 1, H - 2, H + TY + 1>([&](int bx, int by) {
-    const int b = by * BX + bx;
-    eval_point(0, b);
-    eval_point(1, b);
-    eval_point(2, b);
-  });
-  const auto p1_ctr = seg<H - 1, H + TX + 1, H - 1, H + TY + 1>([&](int bx, int by) {
-    const int b = by * BX + bx;
-    const T* V = sZ[0];
-    const T* X = sZ[1];
-    const T* Y = sZ[2];
-    // z_ij = [36 zbar - 4 (X_{i-1,j} + X_ij + Y_{i,j-1} + Y_ij) - (four corners)] / 16
-    const T c = (T(36) * sU[b] - T(4) * ((X[b - 1] + X[b]) + (Y[b - BX] + Y[b])) -
-                 ((V[b - BX - 1] + V[b - BX]) + (V[b - 1] + V[b]))) * T(0.0625);
-    sZ[3][b] = c;
-    eval_point(3, b);
-  });
-  if constexpr (BLEND) {
-    if (!A.blend_external) {
-      // s~_l = |u_- - 2u + u_+| / (|u_-| + 2|u| + |u_+| + 1e-13) (Section 5.1.3); kept
-      // temporarily in the TC arrays
-      for_segs<NT>(p1_qu, p1_pts, p1_ctr, seg<1, BX - 1, 1, BY - 1>([&](int bx, int by) {
-                     const int b = by * BX + bx;
-                     const T u = sU[b];
-                     const T au2 = T(2) * tabs(u);
-                     sTC1[b] = tabs(sU[b - 1] - T(2) * u + sU[b + 1]) /
-                               (tabs(sU[b - 1]) + au2 + tabs(sU[b + 1]) + T(1e-13));
-                     sTC2[b] = tabs(sU[b - BX] - T(2) * u + sU[b + BX]) /
-                               (tabs(sU[b - BX]) + au2 + tabs(sU[b + BX]) + T(1e-13));
-                   }));
+  // (a copy of the phase per diffusion kind: see with_diff)
+  with_diff(m, [&](auto kc) {
+    const auto p1_qu = seg<0, BX, 0, BY>([&](int bx, int by) {
+      const int k = by * BX + bx;
+      const T u = sU[k];
+      if constexpr (FLUX == FLUX_BURGERS) {
+        sQU[k] = flux<FLUX, T>(m, 0, u);
+      } else if constexpr (FLUX == FLUX_BL) {
+        const BLVals<T> r = bl_eval<T>(m, u);
+        sQU[k] = r.f[0];
+        if constexpr (PS::F2) sQU[BN + k] = r.f[1];
+        sQU[PS::DOFF * BN + k] = r.d[0];
+        sQU[(PS::DOFF + 1) * BN + k] = r.d[1];
+      }
+      sQU[(L::NQU - 1) * BN + k] = apot_as<decltype(kc)::value, T>(m, u);
+    });
+    const auto p1_pts = seg<H - 2, H + TX + 1, H - 2, H + TY + 1>([&](int bx, int by) {
+      const int b = by * BX + bx;
+      eval_point(kc, 0, b);
+      eval_point(kc, 1, b);
+      eval_point(kc, 2, b);
+    });
+    const auto p1_ctr = seg<H - 1, H + TX + 1, H - 1, H + TY + 1>([&](int bx, int by) {
+      const int b = by * BX + bx;
+      const T* V = sZ[0];
+      const T* X = sZ[1];
+      const T* Y = sZ[2];
+      // z_ij = [36 zbar - 4 (X_{i-1,j} + X_ij + Y_{i,j-1} + Y_ij) - (four corners)] / 16
+      const T c = (T(36) * sU[b] - T(4) * ((X[b - 1] + X[b]) + (Y[b - BX] + Y[b])) -
+                   ((V[b - BX - 1] + V[b - BX]) + (V[b - 1] + V[b]))) * T(0.0625);
+      sZ[3][b] = c;
+      eval_point(kc, 3, b);
+    });
+    if constexpr (BLEND) {
+      if (!A.blend_external) {
+        // s~_l = |u_- - 2u + u_+| / (|u_-| + 2|u| + |u_+| + 1e-13) (Section 5.1.3); kept
+        // temporarily in the TC arrays
+        for_segs<NT>(p1_qu, p1_pts, p1_ctr, seg<1, BX - 1, 1, BY - 1>([&](int bx, int by) {
+                       const int b = by * BX + bx;
+                       const T u = sU[b];
+                       const T au2 = T(2) * tabs(u);
+                       sTC1[b] = tabs(sU[b - 1] - T(2) * u + sU[b + 1]) /
+                                 (tabs(sU[b - 1]) + au2 + tabs(sU[b + 1]) + T(1e-13));
+                       sTC2[b] = tabs(sU[b - BX] - T(2) * u + sU[b + BX]) /
+                                 (tabs(sU[b - BX]) + au2 + tabs(sU[b + BX]) + T(1e-13));
+                     }));
+      } else {
+        for_segs<NT>(p1_qu, p1_pts, p1_ctr);
+      }
     } else {
       for_segs<NT>(p1_qu, p1_pts, p1_ctr);
     }
-  } else {
-    for_segs<NT>(p1_qu, p1_pts, p1_ctr);
-  }
+  });
   __syncthreads();
 
   // ---- P2: high-order residuals, Simpson fluxes, DC potentials, LLF fluxes -------------
