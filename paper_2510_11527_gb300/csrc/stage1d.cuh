@@ -84,16 +84,17 @@ __device__ __forceinline__ T nodc_d2(const T z[5], const T k[5]) {
 __device__ __forceinline__ double d_of(double v) { return v; }
 __device__ __forceinline__ double d_of(float v) { return f2d_exact(v); }
 
-// The launch's scalars, formed once per CTA by one thread: GB300 runs FP64 arithmetic,
-// FP64 compares and double <-> float conversions on its FP64 unit at 1/64 of the FP32
-// rate, so per-thread copies would cost each cell as much as its own FP64 work.
+// The launch's scalars, formed once per tile: GB300 runs FP64 arithmetic, FP64 compares
+// and double <-> float conversions on its FP64 unit at 1/64 of the FP32 rate, so
+// per-thread copies would cost each cell as much as its own FP64 work. Value k of output o
+// comes from lane k; of a mesh's values (C_UMIN on) output 0's copy is read.
 template <class T>
 struct Scal1D {
-  T umin, umax, ih, i6h, i3h2, g, i4hh, i2h;
-  T taut[2], m2[2], n2[2], k6[2], q6[2], cAt[2], cFt[2];
-  double mu[2], nu[2];
-  int comb[2];
+  T t[2][32];
+  double d[2][4];   // C_MU, C_NU unrounded
 };
+enum : int { C_TAU = 0, C_MU, C_NU, C_M2, C_N2, C_K6, C_Q6, C_CA, C_CF, C_UMIN = 16, C_UMAX, C_IH, C_I6H, C_I3H2,
+             C_G, C_I4HH, C_I2H };
 
 // shared memory of one tile
 template <class T, int BX>
@@ -124,8 +125,10 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
   // mesh's values): GB300's FP64 unit takes as long for a warp instruction with one
   // active lane as with 32. Lane l evaluates fl(fl(fl(x y1) y2) y3) with the factors of
   // its value's formula (a factor 1 is exact, so each value is rounded as its formula
-  // is; the divided line scales come from the host); only the stores differ between
-  // lanes.
+  // is; the divided line scales come from the host) and stores it at its own index (a
+  // switch over the lanes' destinations ran its 17 cases one after the other, in the chain
+  // that every stage of a short mesh starts with: 200 cells FP64 35.0 -> 33.0 us per step
+  // on its own, 5000 43.2 -> 37.1).
   for (int o = tid >> 5; o < A.nout; o += NT / 32) {
     const int l = tid & 31;
     const double ih = A.inv_h1, tau = A.tcoef[o] * dtv;
@@ -155,30 +158,11 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
       y2 = l == 22 ? ih : 1.0;
     }
     const double d = ((x * y1) * y2) * y3;
-    const T dt = T(d);
-    switch (o == 0 || l < 16 ? l : 31) {
-      case 0: sc.taut[o] = dt; sc.comb[o] = !is_zero_bits(A.cA[o]); break;
-      case 1: sc.mu[o] = d; break;
-      case 2: sc.nu[o] = d; break;
-      case 3: sc.m2[o] = dt; break;
-      case 4: sc.n2[o] = dt; break;
-      case 5: sc.k6[o] = dt; break;
-      case 6: sc.q6[o] = dt; break;
-      case 7: sc.cAt[o] = dt; break;
-      case 8: sc.cFt[o] = dt; break;
-      case 16: sc.umin = dt; break;
-      case 17: sc.umax = dt; break;
-      case 18: sc.ih = dt; break;
-      case 19: sc.i6h = dt; break;
-      case 20: sc.i3h2 = dt; break;
-      case 21: sc.g = dt; break;
-      case 22: sc.i4hh = dt; break;
-      case 23: sc.i2h = dt; break;
-      default: break;
-    }
+    sc.t[o][l] = T(d);
+    if (l < 4) sc.d[o][l] = d;
   }
   tile_sync<NT>();
-  const T umin = sc.umin, umax = sc.umax;
+  const T umin = sc.t[0][C_UMIN], umax = sc.t[0][C_UMAX];
   const bool blend = A.blend != 0;
   const bool ext = A.blend == 2;
   const bool nodc = A.nodc != 0;
@@ -212,7 +196,7 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
     }
   }
   tile_sync<NT>();
-  const T ih = sc.ih, i6h = sc.i6h, i3h2 = sc.i3h2;
+  const T ih = sc.t[0][C_IH], i6h = sc.t[0][C_I6H], i3h2 = sc.t[0][C_I3H2];
   // points updated by this thread: its own u_{i+1/2} and, in the first tile of a bounded
   // interval, thread 0 also the left end point u_{-1/2} (held at the boundary value
   // when the end is Dirichlet)
@@ -267,7 +251,7 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
   tile_sync<NT>();
   T rP[2] = {rH[0], rH[1]};
   if (blend) {
-    const T g = sc.g;
+    const T g = sc.t[0][C_G];
     for (int b = H - 1 + tid; b <= H + TX; b += NT) {
       sTD[b] = exp(-g * sS[b]);
       if (b < H + TX) sTC[b] = exp(-g * (T(0.5) * (sS[b] + sS[b + 1])));
@@ -282,7 +266,7 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
       const T zm = sU[b], z0 = sP[b], zp = sU[b + 1];
       const T Fr = T(0.5) * (fP[b] + fU[b + 1]) - T(0.5) * alpha_interval<FLUX, T>(m, XD, z0, zp) * (zp - z0);
       const T Fl = T(0.5) * (fU[b] + fP[b]) - T(0.5) * alpha_interval<FLUX, T>(m, XD, zm, z0) * (z0 - zm);
-      const T RL = (aU[b + 1] - T(2) * aP[b] + aU[b]) * sc.i4hh - (Fr - Fl) * sc.i2h;
+      const T RL = (aU[b + 1] - T(2) * aP[b] + aU[b]) * sc.t[0][C_I4HH] - (Fr - Fl) * sc.t[0][C_I2H];
       rP[q] = sTC[b] * rH[q] + (T(1) - sTC[b]) * RL;
     }
     tile_sync<NT>();
@@ -292,9 +276,10 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
   T* Flim = A.limiter ? sFlim : sFH;
   T* Alim = A.limiter ? sAlim : sAH;
   for (int o = 0; o < A.nout; ++o) {
-    const double mu = sc.mu[o], nu = sc.nu[o];
+    const double mu = sc.d[o][C_MU], nu = sc.d[o][C_NU];
+    const bool comb = !is_zero_bits(A.cA[o]);
     if (A.limiter) {
-      const T m2 = sc.m2[o], n2 = sc.n2[o];
+      const T m2 = sc.t[o][C_M2], n2 = sc.t[o][C_N2];
       for (int b = H - 2 + tid; b <= H + TX + 1; b += NT) {
         const T u = sU[b], f = fU[b], a = aU[b];
         if (!nodc) {
@@ -310,7 +295,7 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
       // face factor 2 * parts (6 with diffusion, 2 without); the total face flux of the
       // form without double conservation takes factor 2 (the average is the mean of
       // u^{L,+} and u^{L,-}, one face correction each)
-      const T k6 = sc.k6[o], q6 = sc.q6[o];
+      const T k6 = sc.t[o][C_K6], q6 = sc.t[o][C_Q6];
       for (int b = H - 1 + tid; b <= H + TX; b += NT) {
         if (b < H + TX) {
           const T fh = sFH[b], fl = sFL[b], dF = fh - fl;
@@ -334,7 +319,7 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
       const size_t g = (size_t)gi;
       double ubfe = A.ub[g] - mu * (d_of(Flim[b]) - d_of(Flim[b - 1]));
       if (!nodc) ubfe += nu * ((d_of(Alim[b + 1]) - 2.0 * d_of(Alim[b])) + d_of(Alim[b - 1]));
-      double ubo = sc.comb[o] ? rk_comb(A.cA[o], A.Aub[o][g], A.cF[o], ubfe) : rk_scale(A.cF[o], ubfe);
+      double ubo = comb ? rk_comb(A.cA[o], A.Aub[o][g], A.cF[o], ubfe) : rk_scale(A.cF[o], ubfe);
       if (A.limiter && A.sg[o]) ubo = safeguard<double>(ubo, m.umin, m.umax, A.tol, A.stats, true);
       A.Oub[o][g] = ubo;
     }
@@ -346,9 +331,9 @@ __device__ __forceinline__ void stage1d_tile(const DevModel& m, const StageArgs2
       if (A.bc == AF_BC_DIRICHLET && (gj == -1 || gj == nx - 1)) {
         po = PT(gj == -1 ? A.bc_left : A.bc_right);
       } else {
-        T p = sP[bq[q]] + sc.taut[o] * rP[q];
+        T p = sP[bq[q]] + sc.t[o][C_TAU] * rP[q];
         if (A.limiter) p = tmin(tmax(p, umin), umax);
-        po = sc.comb[o] ? PT(rk_comb(sc.cAt[o], T(A.AV[o][g]), sc.cFt[o], p)) : PT(rk_scale(sc.cFt[o], p));
+        po = comb ? PT(rk_comb(sc.t[o][C_CA], T(A.AV[o][g]), sc.t[o][C_CF], p)) : PT(rk_scale(sc.t[o][C_CF], p));
         if (A.limiter && A.sg[o]) po = safeguard<PT>(po, PT(umin), PT(umax), A.tol, A.stats);
       }
       A.OV[o][g] = po;
