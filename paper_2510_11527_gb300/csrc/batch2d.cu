@@ -337,7 +337,7 @@ af_status build_work(af_batch* b) {
   // mesh (12 resident warps per SM for Buckley-Leverett and the blend, else 16)
   {
     const bool heavy = b->blend || b->flux == AF_FLUX_BL;
-    b->stream_S = af::strip_plan(heavy ? af::MARCH_HEAVY : af::MARCH_LIGHT, [&](int S) {
+    b->stream_S = af::strip_plan(heavy ? af::MARCH_HEAVY : af::MARCH_ITEMS, [&](int S) {
       long long n = 0;
       for (int k = 0; k < b->n; ++k)
         n += (long long)((b->h_inst[k].nx + af::BATCH_STREAM_BAND - 1) / af::BATCH_STREAM_BAND) *

@@ -7,10 +7,12 @@
 // warm-up, but a strip along a front, where the limiter works, lasts past all others
 // (degenerate Burgers 2048^2, per step: 0.44 ms with 16 to 26 rows, 0.48 with 32, 0.56 with
 // 64 in one wave). The heavy kernels' strips are alike, so for them whole waves count (the
-// busiest SM's CTAs, R at a time) as much as the work (blended Buckley-Leverett 2048^2: 28
-// rows, 3.0 waves, 1.14 ms; 26 rows 1.26 ms). Measured per stage against the fixed number of
-// waves used before: Burgers 100^2 23 -> 12 us, 512^2 25 -> 17 us; Buckley-Leverett 1024^2
-// 101 -> 54 us (with its loop-free wave speeds).
+// busiest SM's CTAs, R at a time) more than the work (blended Buckley-Leverett 2048^2: 28
+// rows, 3.0 waves, 1.14 ms; 26 rows 1.26 ms; 4096^2: 84 rows 3.94, 56 rows 4.03 ms), and
+// for a batch's items as much (16 meshes, 5.6 million cells, one step: 29 rows 617, 23 rows
+// 642 us). Measured per stage against the fixed number of waves used before: Burgers 100^2
+// 23 -> 12 us, 512^2 25 -> 17 us; Buckley-Leverett 1024^2 101 -> 54 us (with its loop-free
+// wave speeds).
 #pragma once
 
 namespace af {
@@ -27,7 +29,8 @@ struct MarchKind {
 };
 constexpr MarchKind MARCH_LIGHT = {4, {1.12, 1.25, 1.50, 1.72}, 0.0, 1.0};   // one column per lane
 constexpr MarchKind MARCH_ZERO = {4, {1.05, 1.18, 1.40, 1.60}, 0.0, 1.0};    // the same, zero flux
-constexpr MarchKind MARCH_HEAVY = {3, {0.68, 0.82, 1.00, 0.0}, 0.5, 0.7};    // Buckley-Leverett, blends (relative)
+constexpr MarchKind MARCH_HEAVY = {3, {0.68, 0.82, 1.00, 0.0}, 0.7, 0.5};    // Buckley-Leverett, blends (relative)
+constexpr MarchKind MARCH_ITEMS = {4, {1.12, 1.25, 1.50, 1.72}, 0.5, 0.5};   // a batch's items, dealt to one wave
 constexpr MarchKind MARCH_PAIR = {3, {1.22, 1.40, 1.69, 0.0}, 0.0, 1.0};     // two columns per lane (zero flux)
 
 // warps(S): how many warps strips of S rows make
