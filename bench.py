@@ -266,9 +266,9 @@ def run_gpu(args):
             "kernels": {"stage_ms_avg": round(statistics.mean(stage_ms), 5), "dt_reduce_ms_avg": round(statistics.mean(dt_ms), 5)},
             "e2e": {"value": round(e2e_value, 1), "unit": UNIT, "h2d_bytes_per_step": bytes_in,
                     "d2h_bytes_per_step": bytes_in},
-            # per step: the CFL rate and its finalisation, one stage launch per stage (and
-            # the plain indicator's pass before each blended stage)
-            "gpu_launches": (nst * (2 if bl else 1) + 2) * args.steps,
+            # per step: the CFL rate (its last block forms the step), one stage launch per
+            # stage (and the plain indicator's pass before each blended stage)
+            "gpu_launches": (nst * (2 if bl else 1) + 1) * args.steps,
             "checks": {"bounds": [lo, hi], "safeguard": stats},
             "clocks": clk.summary(),
             "wall_s": round(wall, 3),

@@ -28,8 +28,9 @@ namespace af {
 // position per lane) for meshes that would otherwise leave most SMs idle: GB300's FP64
 // unit passes 2 lanes per clock and SM, so a short mesh is bound by the FP64 rate of the
 // few SMs it runs on. Launched steps of Example 6.5's problem, FP64, 256-cell tiles /
-// one-warp tiles: 200 cells 57 / 43 us, 10,000 61 / 43 us, 38,000 66 / 49 us; beyond
-// 152 x 256 cells the long tile, whose halo costs 2 % of the work instead of 23 %.
+// one-warp tiles: 200 cells 57 / 43 us, 10,000 61 / 43 us, 38,000 66 / 49 us (when the
+// scalars were stored by a switch, which cost both); beyond 152 x 256 cells the long tile,
+// whose halo costs 2 % of the work instead of 23 %.
 template <int TX_, int NT_>
 struct Tile1D {
   static constexpr int TX = TX_, NT = NT_, H = 3, BX = TX + 2 * H;
@@ -369,8 +370,8 @@ __global__ void __launch_bounds__(32) stage1d_warp_kernel(const DevModel m, cons
 // cluster of 8 CTAs takes up to `nsteps` whole steps: warp w of CTA r works on tile
 // r + 8 w (26 cells), every stage ends in a cluster barrier (hardware, no spinning), the
 // CFL maximum is exchanged through distributed shared memory, and each CTA forms the same
-// step from it: 31 us per step, now the chain of ~1300 instructions of one tile per stage.
-// Up to 832 cells a step costs the same; launched stages of one-warp tiles take 43 us.
+// step from it: 28 us per step, now the chain of ~1300 instructions of one tile per stage.
+// Up to 832 cells a step costs the same; launched stages of one-warp tiles take 37 us.
 template <int FLUX, class T, class PT>
 __global__ void __launch_bounds__(32 * MARCH_WARPS) march1d_kernel(const DevModel m,
                                                                    const __grid_constant__ MarchArgs<PT> M) {
