@@ -26,10 +26,11 @@
 //
 // Measured (porous medium; against the four kernels with 19 scratch arrays, which the blend
 // and, where they are faster, FP64 meshes still take: march3d_takes): FP32-mixed 128^3
-// SSP-RK3 step 1.90 -> 0.51 ms, FP64 80^3 SSP-RK(5,4) step 3.36 -> 2.55 ms. FP64 is bound by the FP64 unit (77 % of its cycles
-// busy), FP32-mixed by instruction issue (about 900 instructions per layer and full row)
-// and the waits of one CTA's 16 warps on each other at the barrier; DRAM moves 58 bytes
-// per cell and stage. With two barriers per step the FP32 step took 0.66 ms.
+// SSP-RK3 step 1.90 -> 0.50 ms, FP64 80^3 SSP-RK(5,4) step 3.36 -> 2.55 ms. FP64 is bound by
+// the FP64 unit (77 % of its cycles busy), FP32-mixed by instruction issue (about 900
+// instructions per layer and full row) and the waits of one CTA's 16 warps on each other at
+// the barrier; DRAM moves 58 bytes per cell and stage. With two barriers per step the FP32
+// step took 0.66 ms.
 #pragma once
 #include "launch.h"
 #include "march3d_plan.h"
