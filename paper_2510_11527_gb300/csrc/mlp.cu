@@ -397,6 +397,15 @@ __device__ __forceinline__ unsigned long long splitmix64(unsigned long long z) {
 // and wait for the completion of the one before
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Load, after grid_dependency_wait, of what an earlier launch may still have been writing
+// when this one started. Such memory changes while the kernel runs, so its pointers are not
+// __restrict__ and it is not read through the read-only path: volatile keeps the load
+// behind the wait, and a relaxed load at device scope sees what the wait made visible.
+__device__ __forceinline__ float load_written(const float* p) {
+  float v;
+  asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
 
 // Forward + backward of a minibatch in FP32 with the tensor-core path's rounding points
 // (bf16 inputs and weights of the two hidden layers): the gradient of the batch-mean loss
@@ -426,7 +435,7 @@ constexpr int TRAIN_ROW = NPARAM + 7;     // 1800 floats per row: gradient, loss
 
 __global__ void __launch_bounds__(256, 2) train_kernel(const float* __restrict__ feat, const float* __restrict__ label,
                                                     long long nsamples, int batch, unsigned long long seed, int step,
-                                                    const float* __restrict__ params, float* __restrict__ partial) {
+                                                    const float* params, float* partial) {
   __shared__ __align__(16) float W1T[NIN][NH], W2T[NH][NH], W2[NH][NH];   // [input][unit], [input][unit], [unit][input]
   __shared__ float b1[NH], b2[NH], w3[NH];
   __shared__ __align__(16) float xT[NIN][TRAIN_LD], h1T[NH][TRAIN_LD], h2T[NH][TRAIN_LD];
@@ -455,18 +464,18 @@ __global__ void __launch_bounds__(256, 2) train_kernel(const float* __restrict__
   };
   if (blockIdx.x < tiles) fetch(blockIdx.x);
   grid_dependency_wait();
-  for (int k = tid; k < NH * NIN; k += 256) W1T[k % NIN][k / NIN] = bfr(params[OFF_W1 + k]);
+  for (int k = tid; k < NH * NIN; k += 256) W1T[k % NIN][k / NIN] = bfr(load_written(params + OFF_W1 + k));
   for (int k = tid; k < NH * NH; k += 256) {
-    const float w = bfr(params[OFF_W2 + k]);
+    const float w = bfr(load_written(params + OFF_W2 + k));
     W2[k / NH][k % NH] = w;
     W2T[k % NH][k / NH] = w;
   }
   if (tid < NH) {
-    b1[tid] = params[OFF_B1 + tid];
-    b2[tid] = params[OFF_B2 + tid];
-    w3[tid] = params[OFF_W3 + tid];
+    b1[tid] = load_written(params + OFF_B1 + tid);
+    b2[tid] = load_written(params + OFF_B2 + tid);
+    w3[tid] = load_written(params + OFF_W3 + tid);
   }
-  const float b3 = params[OFF_B3];
+  const float b3 = load_written(params + OFF_B3);
   // this thread's gradient entries: W2 (unit go, inputs gq + 8 k), W1 (unit go, inputs
   // gq + 8 k < 21) and one entry of b1, b2, w3 or b3
   const int go = tid >> 3, gq = tid & 7;
@@ -590,13 +599,13 @@ __global__ void __launch_bounds__(256, 2) train_kernel(const float* __restrict__
 // sum over the CTAs' rows of column q = 32 blockIdx + lane (the gradient entries, then the
 // loss at NPARAM) in a fixed order: warp w takes rows w, w + 8, ..., then the warps in
 // order; valid in warp 0
-__device__ __forceinline__ float column_sum(const float* __restrict__ partial, int rows) {
+__device__ __forceinline__ float column_sum(const float* partial, int rows) {
   __shared__ float sm[8][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = blockIdx.x * 32 + lane;
   float acc = 0.f;
   if (q <= NPARAM) {
 #pragma unroll 16
-    for (int r = warp; r < rows; r += 8) acc += partial[(size_t)r * TRAIN_ROW + q];
+    for (int r = warp; r < rows; r += 8) acc += load_written(partial + (size_t)r * TRAIN_ROW + q);
   }
   sm[warp][lane] = acc;
   __syncthreads();
@@ -608,10 +617,9 @@ constexpr int COLUMN_CTAS = (NPARAM + 1 + 31) / 32;
 
 // Adam on the FP32 master weights with the gradient summed over the CTAs' rows; refreshes
 // the bf16 copies
-__global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ p, float* __restrict__ m,
-                                                   float* __restrict__ v, const float* __restrict__ partial, int rows,
+__global__ void __launch_bounds__(256) adam_kernel(float* p, float* m, float* v, const float* partial, int rows,
                                                    float lr, float c1, float c2, __nv_bfloat16* w1q,
-                                                   __nv_bfloat16* w2q, float* __restrict__ loss) {
+                                                   __nv_bfloat16* w2q, float* loss) {
   launch_dependents();
   grid_dependency_wait();
   const float g = column_sum(partial, rows);
@@ -621,18 +629,17 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ p, float*
     *loss = g;
     return;
   }
-  const float mq = 0.9f * m[q] + 0.1f * g, vq = 0.999f * v[q] + 0.001f * g * g;
+  const float mq = 0.9f * load_written(m + q) + 0.1f * g, vq = 0.999f * load_written(v + q) + 0.001f * g * g;
   m[q] = mq;
   v[q] = vq;
-  const float w = p[q] - lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
+  const float w = load_written(p + q) - lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
   p[q] = w;
   if (q < OFF_B1) w1q[(q / NIN) * 32 + q % NIN] = __float2bfloat16_rn(w);
   else if (q >= OFF_W2 && q < OFF_B2) w2q[q - OFF_W2] = __float2bfloat16_rn(w);
 }
 
 // the summed gradient (and the loss at NPARAM) alone
-__global__ void __launch_bounds__(256) grad_kernel(const float* __restrict__ partial, int rows,
-                                                   float* __restrict__ grad) {
+__global__ void __launch_bounds__(256) grad_kernel(const float* partial, int rows, float* grad) {
   const float g = column_sum(partial, rows);
   const int q = blockIdx.x * 32 + (int)threadIdx.x;
   if (threadIdx.x < 32 && q <= NPARAM) grad[q] = g;

@@ -204,6 +204,27 @@ def test_gradient_at_tile_edges(n):
     assert loss == loss2 and np.array_equal(g, g2)
 
 
+@pytest.mark.parametrize("n", [1, 4096, 32 * 304 + 5])
+def test_overlapping_steps_equal_single_steps(n):
+    """The launches of one call overlap, each one's start with the end of the one before;
+    the first launch of a call does not. 24 steps in one call and 24 calls of one step are
+    the same arithmetic, so the parameters are the same bit for bit (batches of one tile,
+    of a tile per CTA, and of more tiles than CTAs)."""
+    from paper_2510_11527_gb300 import capi
+    rng = np.random.default_rng(n)
+    xd = torch.from_numpy(rng.normal(0, 0.6, (n, 21)).astype(np.float32)).cuda()
+    yd = torch.from_numpy(rng.uniform(0, 1, n).astype(np.float32)).cuda()
+    out = []
+    for calls in (1, 24):
+        net, _ = _net(9)
+        try:
+            losses = [capi.af_mlp_train(net, xd.data_ptr(), yd.data_ptr(), n, n, 24 // calls, 3e-3, 0) for _ in range(calls)]
+            out.append((capi.af_mlp_get_params(net), losses[-1]))
+        finally:
+            capi.af_mlp_destroy(net)
+    assert np.array_equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
+
+
 def _training_data(count=8, n=128, steps=4):
     """Method-labelled patches: random piecewise-constant fields advanced a few steps by
     the plain method (Buckley-Leverett, FP32-mixed, plain blend)."""
