@@ -35,6 +35,13 @@ __device__ __forceinline__ unsigned crit_flags(const DevModel& m, int dir, doubl
   return f;
 }
 
+// bits of a rate (never negative), ordered as the rate, a NaN of either sign above all. The
+// sign is cleared in the high word: a mask of all 64 bits is compiled as the FP64 unit's
+// absolute value, which leaves a NaN's sign as it was.
+__device__ __forceinline__ unsigned long long rate_bits_of(double r) {
+  return ((unsigned long long)(unsigned)(__double2hiint(r) & 0x7FFFFFFF) << 32) | (unsigned)__double2loint(r);
+}
+
 // rate over the flagged extrema (see dt_rate_kernel)
 __device__ __forceinline__ double crit_rate(const DevModel& m, int dim, double inv_h1, double inv_h2, double kmax,
                                             unsigned long long flags, double rate) {
@@ -145,7 +152,7 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
                                                                unsigned long long* rate_bits, int bc, double gl,
                                                                double gr, const DtFinal fin) {
   static_assert(FLUX == FLUX_BL, "the other fluxes take dt_rate_maxu_kernel");
-  double best = 0.0;
+  unsigned long long best = 0ull;   // magnitude bits of the largest rate
   unsigned flags = 0u;
   const double kd1 = kmax * inv_h1 * inv_h1, kd2 = kmax * inv_h2 * inv_h2;
   const bool rect = dim == 2 && bc != AF_BC_PERIODIC;
@@ -155,12 +162,15 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
   // for the cells whose estimate is within 2^-12 of the block's largest estimate: the
   // cell with the largest FP64 rate is always among them, so the maximum is the same.
   // (Finding each cell's coordinates by 64-bit divisions, and estimating every cell twice,
-  // had cost most of the kernel: 0.28 ms per step at 4096^2.)
+  // had cost most of the kernel: 0.28 ms per step at 4096^2.) An estimate that overflows or
+  // is NaN (a NaN average, an average too large for FP32) compares as larger than all
+  // others: estimates are reduced by their magnitude bits, the threshold of such a block is
+  // NaN and all of its cells are looked at in FP64.
   auto rate64 = [&](double u) {
     const BLVals<double> r = bl_eval<double>(m, u);
     double b = r.d[dim == 1 ? 1 : 0] * inv_h1 + kd1;
     if (dim == 2) b = tmax(b, r.d[1] * inv_h2 + kd2);
-    return b;
+    return rate_bits_of(b);
   };
   const float ih1f = (float)inv_h1, ih2f = (float)inv_h2, kd1f = (float)kd1, kd2f = (float)kd2;
   auto rate32 = [&](double u) {
@@ -169,6 +179,7 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
     if (dim == 2) b = fmaxf(b, r.d[1] * ih2f + kd2f);
     return b;
   };
+  auto mag32 = [](float v) { return __float_as_uint(v) & 0x7FFFFFFFu; };   // ordered as |v|, NaN above all
   // cells in segments of up to RATE_SEG columns of a row, so that a thread's cells need no
   // division to find their coordinates
   constexpr int RATE_SEG = 4 * RED_THREADS;
@@ -184,14 +195,16 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
     }
   };
   auto bits_of = [](double u) { return (unsigned long long)__double_as_longlong(u); };
-  float m32 = 0.0f;
+  unsigned m32 = 0u;   // magnitude bits of the largest estimate
   {
-    unsigned long long last = ~0ull;   // bits of the last u evaluated (NaN: none)
+    unsigned long long last = 0ull;   // bits of the last u evaluated
+    bool any = false;
     cells([&](int i, int j, size_t k) {
       const double u = ub[k];
-      if (bits_of(u) != last) {
-        m32 = fmaxf(m32, rate32(u));
+      if (!any || bits_of(u) != last) {
+        m32 = max(m32, mag32(rate32(u)));
         last = bits_of(u);
+        any = true;
       }
       // an extremum lies strictly inside a face's interval only if its ends differ
       double un = ub[(size_t)j * nx + (i + 1 == nx ? 0 : i + 1)];
@@ -206,33 +219,33 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
     });
   }
   {
-    const float mine = m32;   // the largest estimate among this thread's cells
-    __shared__ float s32[RED_THREADS / 32];
-    for (int o = 16; o > 0; o >>= 1) m32 = fmaxf(m32, __shfl_xor_sync(0xffffffffu, m32, o));
+    const float mine = __uint_as_float(m32);   // the largest estimate among this thread's cells
+    __shared__ unsigned s32[RED_THREADS / 32];
+    m32 = __reduce_max_sync(0xffffffffu, m32);
     if ((threadIdx.x & 31) == 0) s32[threadIdx.x >> 5] = m32;
     __syncthreads();
-    for (int w = 0; w < RED_THREADS / 32; ++w) m32 = fmaxf(m32, s32[w]);
-    const float thr = m32 - m32 * (1.0f / 4096.0f);
-    if (mine >= thr) {   // only threads with a candidate look at their cells again
-      unsigned long long last = ~0ull;
-      double lastr = 0.0;
+    for (int w = 0; w < RED_THREADS / 32; ++w) m32 = max(m32, s32[w]);
+    const float top = __uint_as_float(m32), thr = top - top * (1.0f / 4096.0f);
+    if (!(mine < thr)) {   // only threads with a candidate look at their cells again (NaN: all)
+      unsigned long long last = 0ull;
+      bool any = false;
       cells([&](int, int, size_t k) {
         const double u = ub[k];
-        if (bits_of(u) == last) return;
+        if (any && bits_of(u) == last) return;
         if (rate32(u) < thr) return;
-        lastr = rate64(u);
         last = bits_of(u);
-        best = tmax(best, lastr);
+        any = true;
+        best = max(best, rate64(u));
       });
     }
   }
   if (dim == 1 && bc == AF_BC_DIRICHLET && blockIdx.x == 0 && threadIdx.x == 0) {
     const double gv[2] = {gl, gr};
-    for (int s = 0; s < 2; ++s) best = tmax(best, bl_eval<double>(m, gv[s]).d[1] * inv_h1 + kd1);
+    for (int s = 0; s < 2; ++s) best = max(best, rate_bits_of(bl_eval<double>(m, gv[s]).d[1] * inv_h1 + kd1));
   }
-  for (int o = 16; o > 0; o >>= 1) best = tmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+  for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
   flags = __reduce_or_sync(0xffffffffu, flags);
-  __shared__ double sm[RED_THREADS / 32];
+  __shared__ unsigned long long sm[RED_THREADS / 32];
   __shared__ unsigned sf[RED_THREADS / 32];
   if ((threadIdx.x & 31) == 0) {
     sm[threadIdx.x >> 5] = best;
@@ -240,13 +253,13 @@ __global__ void __launch_bounds__(RED_THREADS) dt_rate_kernel(const DevModel m, 
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double b = sm[0];
+    unsigned long long b = sm[0];
     unsigned f = sf[0];
     for (int w = 1; w < RED_THREADS / 32; ++w) {
-      b = tmax(b, sm[w]);
+      b = max(b, sm[w]);
       f |= sf[w];
     }
-    atomicMax(rate_bits, (unsigned long long)__double_as_longlong(b));
+    atomicMax(rate_bits, b);
     if (f) atomicOr(rate_bits + 1, (unsigned long long)f);
     dt_finish(rate_bits, m, fin);
   }

@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(32 * MARCH_WARPS) march1d_kernel(const DevMode
           double d;
           if constexpr (FLUX == FLUX_BL) d = bl_eval<double>(m, v).d[1];
           else d = alpha_interval<FLUX, double>(m, 0, v, v);
-          return (unsigned long long)__double_as_longlong(d * ih + kd);
+          return rate_bits_of(d * ih + kd);
         };
         bits = rate(u);
         if (A0.bc == AF_BC_DIRICHLET && (i == 0 || i == nx - 1)) {   // the end faces' ghosts (nx >= 4)
