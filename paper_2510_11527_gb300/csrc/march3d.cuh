@@ -18,15 +18,15 @@
 // and yz-edges; the 8 corners), each built from sums along one axis after another: 19
 // additions and 8 operations per direction instead of 27 weighted terms per direction.
 //
-// FP32-mixed form: the averages' update keeps the accuracy of FP64 without its unit. The
-// differences of the FP32 face fluxes and potentials are formed without rounding error
-// (TwoSum), multiplied by mu and nu held as FP32 pairs (two products by FMA) and summed
-// with compensation, so the increment carries about 46 bits; it is widened once and added
-// to the FP64 average.
+// FP32-mixed form: stencils and limiters in FP32; the averages are updated from the widened
+// face values in FP64 (differences, products with mu and nu, sums). That costs: with the
+// increment as FP32 pairs, which hold 46 bits of it and lose them for states near FP32's
+// smallest normals, a step of the porous medium at 128^3 took 503 instead of 531 us and one of
+// Burgers' equation with constant diffusion 742 instead of 824 us.
 //
 // Measured (porous medium; against the four kernels with 19 scratch arrays, which the blend
 // and, where they are faster, FP64 meshes still take: march3d_takes): FP32-mixed 128^3
-// SSP-RK3 step 1.90 -> 0.50 ms, FP64 80^3 SSP-RK(5,4) step 3.36 -> 2.55 ms. FP64 is bound by
+// SSP-RK3 step 1.90 -> 0.53 ms, FP64 80^3 SSP-RK(5,4) step 3.36 -> 2.55 ms. FP64 is bound by
 // the FP64 unit (77 % of its cycles busy), FP32-mixed by instruction issue (about 900
 // instructions per layer and full row) and the waits of one CTA's 16 warps on each other at
 // the barrier; DRAM moves 58 bytes per cell and stage. With two barriers per step the FP32
@@ -41,8 +41,7 @@ namespace af {
 // the launch's scalars
 template <class T>
 struct M3Scal {
-  double mu[3], nu[3];                // FP64 form
-  float muh[3], mul[3], nuh[3], nul[3];   // FP32-mixed: the same as FP32 pairs
+  double mu[3], nu[3];
   T mu6[3], nu6[3], kc[3], kd[3];     // 6 mu, 6 nu, (18 or 6) mu, 18 nu
   T taut, umin, umax, cAt, cFt;
   T mid;                              // -30 sum_l 1 / (3 h_l^2)
@@ -66,11 +65,10 @@ __device__ __forceinline__ void m3_scalars(const DevModel& m, const StageArgs3D<
   }
   const double d = ((x * y1) * y2) * y3;
   const T t = T(d);
-  const float h = (float)d, lo = (float)(d - (double)h);
   if (l < 18) {
     switch (kind) {
-      case 0: sc.mu[dir] = d; sc.muh[dir] = h; sc.mul[dir] = lo; break;
-      case 1: sc.nu[dir] = d; sc.nuh[dir] = h; sc.nul[dir] = lo; break;
+      case 0: sc.mu[dir] = d; break;
+      case 1: sc.nu[dir] = d; break;
       case 2: sc.mu6[dir] = t; break;
       case 3: sc.nu6[dir] = t; break;
       case 4: sc.kc[dir] = t; break;
@@ -88,44 +86,48 @@ __device__ __forceinline__ void m3_scalars(const DevModel& m, const StageArgs3D<
   }
 }
 
-// increment of a cell average: FP64, or an FP32 pair
-template <class T> struct Incr;
-template <> struct Incr<double> {
+// exact widening of a stencil value, the FP32 one with integer operations (f2d_exact) but
+// with the test for subnormal values made once for three of them
+__device__ __forceinline__ double m3_wide(float f) {   // zero or normal
+  const unsigned u = __float_as_uint(f), mag = u & 0x7FFFFFFFu;
+  return __hiloint2double((int)(mag == 0u ? u : (u & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ void m3_wide3(const double (&x)[3], double (&y)[3]) {
+  for (int k = 0; k < 3; ++k) y[k] = x[k];
+}
+__device__ __forceinline__ void m3_wide3(const float (&x)[3], double (&y)[3]) {
+  unsigned t = 0xFFFFFFFFu;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    y[k] = m3_wide(x[k]);
+    t = min(t, (__float_as_uint(x[k]) & 0x7FFFFFFFu) - 1u);
+  }
+  if (t < 0x007FFFFFu) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) y[k] = f2d_exact(x[k]);
+  }
+}
+
+// increment of a cell average, in FP64 whatever the stencil type: the two cells of a face
+// take its value with the same rounding
+template <class T>
+struct Incr {
   double v;
   __device__ __forceinline__ void zero() { v = 0.0; }
   // - mu (f0 - fm)
-  __device__ __forceinline__ void conv(const M3Scal<double>& k, int l, double f0, double fm) { v = __fma_rn(-k.mu[l], f0 - fm, v); }
+  __device__ __forceinline__ void conv(const M3Scal<T>& k, int l, T f0, T fm) {
+    const T x[3] = {f0, fm, T(0)};
+    double y[3];
+    m3_wide3(x, y);
+    v = __fma_rn(-k.mu[l], y[0] - y[1], v);
+  }
   // nu (ap - 2 a0 + am)
-  __device__ __forceinline__ void diff(const M3Scal<double>& k, int l, double ap, double a0, double am) {
-    v = __fma_rn(k.nu[l], __fma_rn(-2.0, a0, ap + am), v);
+  __device__ __forceinline__ void diff(const M3Scal<T>& k, int l, T ap, T a0, T am) {
+    const T x[3] = {ap, a0, am};
+    double y[3];
+    m3_wide3(x, y);
+    v = __fma_rn(k.nu[l], __fma_rn(-2.0, y[1], y[0] + y[2]), v);
   }
-  __device__ __forceinline__ double value() const { return v; }
-};
-template <> struct Incr<float> {
-  float h, l;
-  __device__ __forceinline__ void zero() { h = l = 0.0f; }
-  // add (ch + cl) (dh + dl), c a coefficient pair
-  __device__ __forceinline__ void add(float ch, float cl, float dh, float dl) {
-    const float p = __fmul_rn(ch, dh);
-    float e = __fmaf_rn(ch, dh, -p);
-    e = __fmaf_rn(ch, dl, e);
-    e = __fmaf_rn(cl, dh, e);
-    float r;
-    two_sum(h, p, h, r);
-    l = __fadd_rn(l, __fadd_rn(r, e));
-  }
-  __device__ __forceinline__ void conv(const M3Scal<float>& k, int d, float f0, float fm) {
-    float s, e;
-    two_sum(fm, -f0, s, e);
-    add(k.muh[d], k.mul[d], s, e);
-  }
-  __device__ __forceinline__ void diff(const M3Scal<float>& k, int d, float ap, float a0, float am) {
-    float s, e, s2, e2;
-    two_sum(ap, am, s, e);
-    two_sum(s, -2.0f * a0, s2, e2);
-    add(k.nuh[d], k.nul[d], s2, __fadd_rn(e, e2));
-  }
-  __device__ __forceinline__ double value() const { return f2d_exact(h) + f2d_exact(l); }
 };
 
 // What a layer leaves for the one above it: sums over its upper plane of z-faces. The FP64
@@ -301,6 +303,10 @@ __global__ void __launch_bounds__(32 * TY, 1)
   const bool mid = row >= 1 && row < TY - 1;      // forms centres and the y-limiter
   const bool full = row >= 2 && row < TY - 2;     // forms everything
   const bool out = full && lane >= 2 && lane < 2 + M3_BAND && xi < n0 && yi < n1;
+  // the FP64 ends of a step's averages, all at its end, would queue at the FP64 unit: half
+  // of a scheduler's warps form theirs at its start (FP32-mixed porous medium 128^3, step
+  // 570 -> 556 us; with a flux, fewer rows and more work between them, it cost registers)
+  const bool early = sizeof(T) == 4 && !CONV && ((row >> 2) & 1);
   const bool lim = A.limiter != 0, comb = !is_zero_bits(A.cA[o]), sg = lim && A.sg[o];
   const unsigned plane = (unsigned)n0 * n1;
   const unsigned qxy = (unsigned)wrapi(yi, n1) * n0 + wrapi(xi, n0);
@@ -331,6 +337,7 @@ __global__ void __launch_bounds__(32 * TY, 1)
   for (int r = zs - 2; r <= ze + 1; ++r) {
     const int par = r & 1;
     U = to_stencil<T>(un);
+    const double uc = un;
     // of the last layer only the averages are read (in FP32 the test costs more than it saves)
     const bool pts = sizeof(T) == 4 || r <= ze;
 #pragma unroll
@@ -356,7 +363,7 @@ __global__ void __launch_bounds__(32 * TY, 1)
       for (int s = 1; s < 8; ++s) Ap[s] = A.Apt[o][s][q1];
     }
     if (outu) {
-      ubj = A.ub[q2];
+      if constexpr (sizeof(T) == 8) ubj = A.ub[q2];
       if (comb) Aub = A.Aub[o][q2];
     }
     pa = ca;
@@ -383,6 +390,21 @@ __global__ void __launch_bounds__(32 * TY, 1)
     }
     __syncthreads();
     const T aU = apot_k<DIFF, T>(m, U);
+    // ---- z-limiter of cell r - 1, averages of layer r - 2
+    T Fz1 = T(0), Az1 = T(0);
+    auto finish = [&]() {
+      m3_limit<FLUX, T>(m, k, lim, 2, U2, U1, U, aU2, aU1, aU, FHz1, AHz1, Fz1, Az1);
+      if (outu) {
+        Incr<T> w = inc2;
+        if constexpr (CONV) w.conv(k, 2, Fz2, Fz3);
+        w.diff(k, 2, Az1, Az2, Az3);
+        const double v = sizeof(T) == 8 ? ubj + w.v : w.v;
+        double ubo = comb ? rk_comb(A.cA[o], Aub, A.cF[o], v) : rk_scale(A.cF[o], v);
+        if (sg) ubo = safeguard<double>(ubo, m.umin, m.umax, A.tol, A.stats, true);
+        A.Oub[o][q2] = ubo;
+      }
+    };
+    if (full && early) finish();
     const bool xy = r >= zs && r < ze;   // x- and y-directions of layer r are needed
     T AHx = T(0), AHz = T(0), FHx = T(0), FHz = T(0), Fy = T(0), Ay = T(0);
     T am2, am3, am6, am7, zm2, zm3, zm6, zm7;   // row below
@@ -537,6 +559,7 @@ __global__ void __launch_bounds__(32 * TY, 1)
       T res[8];
       Incr<T> inc;
       inc.zero();
+      if constexpr (sizeof(T) == 4) inc.v = uc;   // the average itself, its terms added in turn
       if (xy) {
         // ---- averages: x part of layer r
         {
@@ -617,18 +640,7 @@ __global__ void __launch_bounds__(32 * TY, 1)
           for (int s = 1; s < 8; ++s) A.Opt[o][s][q1] = po[s];
         }
       }
-      // ---- z-limiter of cell r - 1, averages of layer r - 2
-      T Fz1, Az1;
-      m3_limit<FLUX, T>(m, k, lim, 2, U2, U1, U, aU2, aU1, aU, FHz1, AHz1, Fz1, Az1);
-      if (outu) {
-        Incr<T> w = inc2;
-        if constexpr (CONV) w.conv(k, 2, Fz2, Fz3);
-        w.diff(k, 2, Az1, Az2, Az3);
-        const double v = ubj + w.value();
-        double ubo = comb ? rk_comb(A.cA[o], Aub, A.cF[o], v) : rk_scale(A.cF[o], v);
-        if (sg) ubo = safeguard<double>(ubo, m.umin, m.umax, A.tol, A.stats, true);
-        A.Oub[o][q2] = ubo;
-      }
+      if (!early) finish();
       Fz3 = Fz2;
       Fz2 = Fz1;
       Az3 = Az2;

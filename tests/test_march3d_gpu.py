@@ -97,3 +97,30 @@ def test_fp32_mixed_conserves_mass(flux, diff):
     # increments are below 1 per cell: 2^-44 each at worst, added up
     assert abs(math.fsum(got.ravel()) - math.fsum(st[0].ravel())) <= got.size * 2.0 ** -44
     assert float(np.max(np.abs(got - st[0]))) > 1e-3
+
+
+@pytest.mark.parametrize("flux", ["zero", "linear"])
+def test_fp32_mixed_averages_are_updated_in_fp64(flux):
+    """A linear problem scaled by 2^-100 has the same roundings: the values (0.5 .. 1 before),
+    potentials and fluxes (coefficients 2^-1 and 2^-2) keep FP32's normal range, with their
+    last places at 2^-126 or above, and FP64 is far from its own. So the result is the
+    unscaled one times 2^-100 bit for bit, if the averages' increment holds FP64: FP32 parts
+    of it would lose their last bits below 2^-149."""
+    spec = box((40, 27, 30), "zero", "const", limiter=False)
+    spec.diff = ("const", (0.5,))
+    if flux == "linear":
+        spec.flux = ("linear", (1.0, -0.5, 0.25))
+    spec.umin, spec.umax = 0.5, 1.0
+    st = [a.numpy() for a in ai.random_state_3d(spec, seed=5, lo=0.5, hi=1.0)]
+    st = [st[0]] + [a.astype(np.float32).astype(np.float64) for a in st[1:]]
+    tau = oracle.dt_cfl(spec, st[0])
+    out = []
+    for scale in (1.0, 2.0 ** -100):
+        spec.umin, spec.umax = 0.5 * scale, scale
+        with solver(spec, prec="fp32_mixed") as s:
+            s.set_state([a * scale for a in st])
+            s.forward_euler(tau)
+            out.append(s.get_state())
+    assert far([out[0][0]], [st[0]]) > 1e-3
+    for a, b in zip(*out):
+        assert np.array_equal(a * 2.0 ** -100, b)
