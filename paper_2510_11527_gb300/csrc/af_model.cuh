@@ -32,9 +32,10 @@ struct DevModel {
   // unit also performs the double->float conversions, so none happen per use)
   float fpf[4], dpf[4], critf[2][8], critvf[2][8];
   // FP32, limiter on: the extrema inside the bounds and their |f_l'| in two fixed slots per
-  // direction (an empty slot lies at infinity, inside no interval); crit_few = 0 when a
-  // direction has more of them or the state may leave the bounds
-  float critf2[2][2], critvf2[2][2];
+  // direction (an empty slot lies at infinity, inside no interval), and the nearest extrema
+  // left out below and above (infinity: none); crit_few = 0 when a direction has more inside
+  // the bounds or the state may leave them
+  float critf2[2][2], critvf2[2][2], crit_below, crit_above;
   int crit_few;
   int pme_e;             // AF_DIFF_PME: the integer exponent p0 (no conversion per use)
   // parts of the convex decomposition of each limited directional state u^{Lim,+-}
@@ -63,13 +64,17 @@ inline void fill_float_params(DevModel& m) {
     }
 }
 
-// after the bounds are known: DevModel::critf2 (a limited state stays inside the bounds up
-// to the safeguard's tolerance -- data outside them are refused -- so an extremum outside
-// them by more is inside no interval of two of its values). 2D only: a 1D end value may
-// lie outside. (Three slots, enough for all extrema on the line without a look at the
-// bounds, cost 6 %: blended Buckley-Leverett step at 4096^2 3.94 / 4.19 ms.)
+// after the bounds are known: DevModel::critf2. A limited state stays inside the bounds up
+// to the safeguard's tolerance, so an extremum outside them by more is normally inside no
+// interval of two of its values; a kernel looks whether its values reach beyond one (a state
+// written in place, or one that the safeguard has reported) and then takes the loop. 2D only:
+// a 1D end value may lie outside. Blended Buckley-Leverett step at 4096^2: 3.94 ms without
+// that look, 3.83 with one per row of a warp, 4.23 with one per interval, 4.19 with three
+// slots, enough for all extrema on the line.
 inline void fill_few_criticals(DevModel& m, bool limiter, int dim) {
   m.crit_few = limiter && dim == 2 ? 1 : 0;
+  m.crit_below = -INFINITY;
+  m.crit_above = INFINITY;
   const double margin = 1e-5 * (fabs(m.umin) > fabs(m.umax) ? fabs(m.umin) : fabs(m.umax));
   for (int d = 0; d < 2; ++d) {
     int n = 0;
@@ -78,7 +83,14 @@ inline void fill_few_criticals(DevModel& m, bool limiter, int dim) {
       m.critvf2[d][k] = 0.0f;
     }
     for (int k = 0; k < m.ncrit[d]; ++k) {
-      if (m.crit[d][k] <= m.umin - margin || m.crit[d][k] >= m.umax + margin) continue;
+      if (m.crit[d][k] <= m.umin - margin) {
+        m.crit_below = fmaxf(m.crit_below, m.critf[d][k]);
+        continue;
+      }
+      if (m.crit[d][k] >= m.umax + margin) {
+        m.crit_above = fminf(m.crit_above, m.critf[d][k]);
+        continue;
+      }
       if (n == 2) {
         m.crit_few = 0;
         break;
@@ -305,7 +317,7 @@ __device__ __forceinline__ T kappa_fn(const DevModel& m, T u) {
 // db = |f_l'(b)|: the end points plus the interior extrema of f_l' that lie strictly
 // inside (their |f_l'| is tabulated in the model).
 template <int FLUX, class T>
-__device__ __forceinline__ T alpha_interval_pre(const DevModel& m, int dir, T a, T b, T da, T db) {
+__device__ __forceinline__ T alpha_interval_pre(const DevModel& m, int dir, T a, T b, T da, T db, bool few = false) {
   if constexpr (FLUX == FLUX_LINEAR) {
     return tabs(par<T>(m.fp, m.fpf, dir));
   } else if constexpr (FLUX == FLUX_BURGERS) {
@@ -316,7 +328,7 @@ __device__ __forceinline__ T alpha_interval_pre(const DevModel& m, int dir, T a,
     if constexpr (sizeof(T) == 4) {
       // the usual case without a loop (two compares and a select per slot): the loop, with
       // its indexed constants, took most of a Buckley-Leverett LLF flux's instructions
-      if (m.crit_few) {
+      if (few) {
 #pragma unroll
         for (int k = 0; k < 2; ++k)
           if ((lo < m.critf2[dir][k]) & (m.critf2[dir][k] < hi)) best = tmax(best, m.critvf2[dir][k]);

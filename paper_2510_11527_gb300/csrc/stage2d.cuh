@@ -344,6 +344,13 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
   const T umin = sc.t[0][S_UMIN], umax = sc.t[0][S_UMAX];
 
   // ---- P1: centres and pointwise nonlinearities ----------------------------------------
+  // FP32 Buckley-Leverett: whether the tile's averages and points reach beyond an extremum
+  // that has no slot (see fill_few_criticals)
+  constexpr bool FEW = FLUX == FLUX_BL && sizeof(T) == 4;
+  bool few = false, beyond = false;
+  auto look = [&](T z) {
+    if constexpr (FEW) beyond |= (z < m.crit_below) | (z > m.crit_above);
+  };
   auto eval_point = [&](auto kc, int type, int b) {
     const T z = sZ[type][b];
     if constexpr (FLUX == FLUX_BURGERS) {
@@ -376,6 +383,7 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
     const auto p1_qu = seg<0, BX, 0, BY>([&](int bx, int by) {
       const int k = by * BX + bx;
       const T u = sU[k];
+      look(u);
       if constexpr (FLUX == FLUX_BURGERS) {
         sQU[k] = flux<FLUX, T>(m, 0, u);
       } else if constexpr (FLUX == FLUX_BL) {
@@ -389,6 +397,7 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
     });
     const auto p1_pts = seg<H - 2, H + TX + 1, H - 2, H + TY + 1>([&](int bx, int by) {
       const int b = by * BX + bx;
+      for (int t = 0; t < 3; ++t) look(sZ[t][b]);
       eval_point(kc, 0, b);
       eval_point(kc, 1, b);
       eval_point(kc, 2, b);
@@ -424,7 +433,8 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
       for_segs<NT>(p1_qu, p1_pts, p1_ctr);
     }
   });
-  __syncthreads();
+  if constexpr (FEW) few = !__syncthreads_or(beyond) && m.crit_few;
+  else __syncthreads();
 
   // ---- P2: high-order residuals, Simpson fluxes, DC potentials, LLF fluxes -------------
   const T i6h1 = sc.t[0][S_I6H1], i6h2 = sc.t[0][S_I6H2];
@@ -522,13 +532,13 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
   const auto p2_fl1 = seg<H - 2, H + TX + 1, H, H + TY>([&](int bx, int by) {
     const int b = by * BX + bx;
     const T ul = sU[b], ur = sU[b + 1];
-    const T al = alpha_interval_pre<FLUX, T>(m, 0, ul, ur, dU(b, 0), dU(b + 1, 0));
+    const T al = alpha_interval_pre<FLUX, T>(m, 0, ul, ur, dU(b, 0), dU(b + 1, 0), few);
     sFL1[b] = T(0.5) * (fU(b, 0) + fU(b + 1, 0)) - T(0.5) * al * (ur - ul);
   });
   const auto p2_fl2 = seg<H, H + TX, H - 2, H + TY + 1>([&](int bx, int by) {
     const int b = by * BX + bx;
     const T ul = sU[b], ur = sU[b + BX];
-    const T al = alpha_interval_pre<FLUX, T>(m, 1, ul, ur, dU(b, 1), dU(b + BX, 1));
+    const T al = alpha_interval_pre<FLUX, T>(m, 1, ul, ur, dU(b, 1), dU(b + BX, 1), few);
     sFL2[b] = T(0.5) * (fU(b, 1) + fU(b + BX, 1)) - T(0.5) * al * (ur - ul);
   });
   if constexpr (BLEND) {
@@ -606,9 +616,9 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
     auto cu = [&](int bb, int dir) -> PV { return PV{sU[bb], fU(bb, dir), aU(bb), dU(bb, dir)}; };
     auto lowres = [&](int dir, const PV& pm, const PV& p0, const PV& pp) -> T {
       const T Fr = T(0.5) * (p0.f + pp.f) -
-                   T(0.5) * alpha_interval_pre<FLUX, T>(m, dir, p0.z, pp.z, p0.d, pp.d) * (pp.z - p0.z);
+                   T(0.5) * alpha_interval_pre<FLUX, T>(m, dir, p0.z, pp.z, p0.d, pp.d, few) * (pp.z - p0.z);
       const T Fl = T(0.5) * (pm.f + p0.f) -
-                   T(0.5) * alpha_interval_pre<FLUX, T>(m, dir, pm.z, p0.z, pm.d, p0.d) * (p0.z - pm.z);
+                   T(0.5) * alpha_interval_pre<FLUX, T>(m, dir, pm.z, p0.z, pm.d, p0.d, few) * (p0.z - pm.z);
       return (pp.a - T(2) * p0.a + pm.a) * (dir == 0 ? i4h21 : i4h22) - (Fr - Fl) * (dir == 0 ? i2h1 : i2h2);
     };
     const int b = cell ? bo : H * BX + H;

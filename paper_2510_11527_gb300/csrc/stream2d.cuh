@@ -68,6 +68,7 @@ struct RowSlot {
   // theta^{d,s}_1 of the cell, low-order residuals of the row's x-lines (V, X, Y)
   T s2, tc1, td1, LV1, LX1, LY1;
   T FVX;   // LLF flux (y) between V of the row below and X of this row
+  bool in;  // FP32 Buckley-Leverett: no value of the warp's row reaches beyond the slots' extrema
 };
 
 // f_l, |f_l'| and a at one value: returns f_1 in f1, f_2 in f2, |f_1'| in d1, |f_2'| in d2
@@ -107,8 +108,8 @@ __device__ __forceinline__ T line_alpha(const DevModel& m, int dir, T z0, T z1, 
 }
 
 template <int FLUX, class T>
-__device__ __forceinline__ T llf(const DevModel& m, int dir, T ul, T ur, T fl, T fr, T dl, T dr, T half) {
-  const T al = alpha_interval_pre<FLUX, T>(m, dir, ul, ur, dl, dr);
+__device__ __forceinline__ T llf(const DevModel& m, int dir, T ul, T ur, T fl, T fr, T dl, T dr, T half, bool few) {
+  const T al = alpha_interval_pre<FLUX, T>(m, dir, ul, ur, dl, dr, few);
   return sfma(-(half * al), ur - ul, half * (fl + fr));
 }
 
@@ -196,6 +197,14 @@ __device__ __forceinline__ void stream_step(const StreamCtx<FLUX, DIFF, T>& c, i
   cur.V = in.V;
   cur.X = in.X;
   cur.Y = in.Y;
+  // whether the intervals between values of this row and the one before hold none but the
+  // slots' extrema (uniform over the warp)
+  bool few = false;
+  if constexpr (BL && sizeof(T) == 4) {
+    cur.in = __all_sync(0xffffffffu, (fmn(min3(cur.V, cur.X, cur.Y), cur.U) >= m.crit_below) &
+                                         (fmx(max3(cur.V, cur.X, cur.Y), cur.U) <= m.crit_above));
+    few = m.crit_few && cur.in && p1.in;
+  }
   const T Xm = shup(cur.X);
   cur.Vm = shup(cur.V);
   // z_ij = [36 zbar - 4 (X_{i-1,j} + X_ij + Y_{i,j-1} + Y_ij) - (four corners)] / 16
@@ -251,11 +260,11 @@ __device__ __forceinline__ void stream_step(const StreamCtx<FLUX, DIFF, T>& c, i
     AH1 = cell_pot<T>(sv, sx, sy, cur.aC, false, k.r36);
     if constexpr (BK != 0) AH1 = blendw(td1, AH1, cur.aU);
   }
-  const T FL1 = llf<FLUX, T>(m, 0, cur.U, Up, f1U, f1Up, d1U, d1Up, half);
+  const T FL1 = llf<FLUX, T>(m, 0, cur.U, Up, f1U, f1Up, d1U, d1Up, half, few);
   // the face on the left, formed here as its owner forms it (same inputs, same code)
-  const T FL1m = llf<FLUX, T>(m, 0, Um, cur.U, f1Um, f1U, d1Um, d1U, half);
+  const T FL1m = llf<FLUX, T>(m, 0, Um, cur.U, f1Um, f1U, d1Um, d1U, half, few);
   // y-face between rows r-1 and r
-  const T FL2 = llf<FLUX, T>(m, 1, p1.U, cur.U, p1.fU, cur.fU, p1.dU, cur.dU, half);
+  const T FL2 = llf<FLUX, T>(m, 1, p1.U, cur.U, p1.fU, cur.fU, p1.dU, cur.dU, half, few);
   // blend: the x-face of row r; theta^{c,s}_2 of the y-face between rows r-1 and r and
   // theta^{d,s}_2 of cell (i, r-1), with the y-face flux and the y cell potential of
   // row r-1 (both first used by this step's y-limiter); the low-order residuals of the
@@ -269,15 +278,15 @@ __device__ __forceinline__ void stream_step(const StreamCtx<FLUX, DIFF, T>& c, i
     p1.AH2 = blendw(td2, p1.AH2, p1.aU);
     // x-lines: V between Y_i and Y_{i+1}, X between the averages of cells i and i+1,
     // Y between V_{i-1} and V_i; F(V_{i-1}, Y_i) is the left lane's F(V, Y_{+1})
-    const T FYV = llf<FLUX, T>(m, 0, cur.Y, cur.V, f1Y, f1V, d1Y, d1V, half);
-    const T FVY = llf<FLUX, T>(m, 0, cur.V, Yp, f1V, f1Yp, d1V, d1Yp, half);
-    const T FUX = llf<FLUX, T>(m, 0, cur.U, cur.X, f1U, f1X, d1U, d1X, half);
-    const T FXU = llf<FLUX, T>(m, 0, cur.X, Up, f1X, f1Up, d1X, d1Up, half);
+    const T FYV = llf<FLUX, T>(m, 0, cur.Y, cur.V, f1Y, f1V, d1Y, d1V, half, few);
+    const T FVY = llf<FLUX, T>(m, 0, cur.V, Yp, f1V, f1Yp, d1V, d1Yp, half, few);
+    const T FUX = llf<FLUX, T>(m, 0, cur.U, cur.X, f1U, f1X, d1U, d1X, half, few);
+    const T FXU = llf<FLUX, T>(m, 0, cur.X, Up, f1X, f1Up, d1X, d1Up, half, few);
     cur.LV1 = lowres_s<T>(FYV, FVY, cur.aY, cur.aV, aYp, kb.i2h1, kb.i4h21);
     cur.LX1 = lowres_s<T>(FUX, FXU, cur.aU, cur.aX, aUp, kb.i2h1, kb.i4h21);
     cur.LY1 = lowres_s<T>(shup(FVY), FYV, cur.aVm, cur.aY, cur.aV, kb.i2h1, kb.i4h21);
     // y-direction flux between V of row r-1 and X of row r (the next step's X-line)
-    cur.FVX = llf<FLUX, T>(m, 1, p1.V, cur.X, p1.fV, cur.fX, p1.dV, cur.dX, half);
+    cur.FVX = llf<FLUX, T>(m, 1, p1.V, cur.X, p1.fV, cur.fX, p1.dV, cur.dX, half, few);
   }
 
   // ---- point residuals: x-lines of row r
@@ -308,9 +317,9 @@ __device__ __forceinline__ void stream_step(const StreamCtx<FLUX, DIFF, T>& c, i
       // y-lines of row r-1: V between X_{r-1} and X_r, X between V_{r-2} and V_{r-1}
       // (F(V_{r-2}, X_{r-1}) formed one step earlier), Y between the averages of rows
       // r-1 and r
-      const T FXV = llf<FLUX, T>(m, 1, p1.X, p1.V, p1.fX, p1.fV, p1.dX, p1.dV, half);
-      const T FUY = llf<FLUX, T>(m, 1, p1.U, p1.Y, p1.fU, p1.fY, p1.dU, p1.dY, half);
-      const T FYU = llf<FLUX, T>(m, 1, p1.Y, cur.U, p1.fY, cur.fU, p1.dY, cur.dU, half);
+      const T FXV = llf<FLUX, T>(m, 1, p1.X, p1.V, p1.fX, p1.fV, p1.dX, p1.dV, half, few);
+      const T FUY = llf<FLUX, T>(m, 1, p1.U, p1.Y, p1.fU, p1.fY, p1.dU, p1.dY, half, few);
+      const T FYU = llf<FLUX, T>(m, 1, p1.Y, cur.U, p1.fY, cur.fU, p1.dY, cur.dU, half, few);
       const T LV2 = lowres_s<T>(FXV, cur.FVX, p1.aX, p1.aV, cur.aX, kb.i2h2, kb.i4h22);
       const T LX2 = lowres_s<T>(p1.FVX, FXV, p2.aV, p1.aX, p1.aV, kb.i2h2, kb.i4h22);
       const T LY2 = lowres_s<T>(FUY, FYU, p1.aU, p1.aY, cur.aU, kb.i2h2, kb.i4h22);

@@ -4,6 +4,7 @@ segment's, row's or mesh's edge; and the speeds of the LLF flux over intervals t
 extrema on either side of zero, with and without the limiter, against the oracle."""
 import numpy as np
 import pytest
+import torch
 
 import af_inputs as ai
 import oracle
@@ -55,3 +56,30 @@ def test_speeds_over_intervals_with_extrema(gravity, limiter, blend):
     # FP32 stencils: the bounds of the other FP32-mixed comparisons (values of order 1)
     assert max(float(np.max(np.abs(np.asarray(g, np.float64) - w))) for g, w in zip(got, want)) <= 1e-5
     assert max(float(np.mean(np.abs(np.asarray(g, np.float64) - w))) for g, w in zip(got, want)) <= 1e-6
+
+
+@pytest.mark.parametrize("gravity", [0.0, 5.0])
+@pytest.mark.parametrize("blend", ["off", "plain"])
+@pytest.mark.parametrize("bc", ["periodic", "outflow"])
+def test_speeds_of_a_state_written_beyond_the_bounds(gravity, blend, bc):
+    """A state written in place can reach beyond the bounds, over extrema of f' that no
+    limited state meets (f_1': 1.366 and -0.366): its speeds are still those of the interval,
+    FP32-mixed as FP64."""
+    from paper_2510_11527_gb300 import Solver
+    spec = ai.Spec(dim=2, nx=61, ny=47, x0=0, x1=1.5, y0=0, y1=1.0, flux=("bl", (gravity,)), diff=("const", (0.01,)),
+                   umin=0.0, umax=1.0, blend=blend, bc=bc)
+    inside = [a.numpy() for a in ai.random_state_2d(spec, seed=7)]
+    got = {}
+    for prec in ("fp64", "fp32_mixed"):
+        rng = np.random.default_rng(3)
+        with Solver(spec, precision=prec) as s:
+            s.set_state(inside)
+            for t in s.device_tensors():
+                t.copy_(torch.from_numpy(rng.uniform(-0.8, 1.8, tuple(t.shape)).astype(np.float32)))
+            torch.cuda.synchronize()
+            s.forward_euler(0.25 * oracle.dt_cfl(spec, inside[0]))
+            got[prec] = s.get_state()
+    # FP32 stencils: the bounds of the other FP32-mixed comparisons (values of order 1)
+    d = [np.abs(a - b) for a, b in zip(got["fp64"], got["fp32_mixed"])]
+    assert max(float(x.max()) for x in d) <= 1e-5
+    assert max(float(x.mean()) for x in d) <= 1e-6
