@@ -30,8 +30,10 @@ inline M3Plan m3_plan(const int* n, int TY) {
   p.S = n[2];
   const long long tiles = (long long)p.bands * p.rows;
   double best = -1.0;
-  for (int s = 1; s <= n[2] && s <= 152 * 8; ++s) {
-    const int L = (n[2] + s - 1) / s;
+  // one number of strips per height (the next one lowers it): about 2 sqrt(n[2]) of them, as
+  // every stage's launch asks (1216 strips one by one took 5 us of host time per call)
+  for (int s = 1, L; s <= n[2] && s <= 152 * 8; s = L > 1 ? (n[2] + L - 2) / (L - 1) : n[2] + 1) {
+    L = (n[2] + s - 1) / s;
     const long long waves = (tiles * ((n[2] + L - 1) / L) + 151) / 152;
     if (best < 0.0 || waves * (L + 1.2) < best) {
       best = waves * (L + 1.2);
