@@ -32,17 +32,20 @@ struct DevModel {
   // unit also performs the double->float conversions, so none happen per use)
   float fpf[4], dpf[4], critf[2][8], critvf[2][8];
   // FP32, limiter on: the extrema inside the bounds and their |f_l'| in two fixed slots per
-  // direction (an empty slot lies at infinity, inside no interval), and the nearest extrema
-  // left out below and above (infinity: none); crit_few = 0 when a direction has more inside
-  // the bounds or the state may leave them
-  float critf2[2][2], critvf2[2][2], crit_below, crit_above;
-  int crit_few;
+  // direction (an empty slot lies at infinity, inside no interval). They serve values between
+  // crit_below and crit_above, the nearest extrema without a slot (infinity: none; no value
+  // at all when a direction has more inside the bounds or the state may leave them)
+  float critf2[2][2], critvf2[2][2];
+  float crit_below;
   int pme_e;             // AF_DIFF_PME: the integer exponent p0 (no conversion per use)
   // parts of the convex decomposition of each limited directional state u^{Lim,+-}
   // (Section 5.1.1, per direction in Section 5.2): 3 -- the face correction and the two
   // potential corrections -- when the equation diffuses, 1 when a(u) is constant and
   // only the face correction is present. The face limiter factor is 2d times this.
   int lim_parts;
+  // (sizeof(DevModel) counts: each warp of the batch's march holds one in shared memory, and
+  // 8 bytes more cost 4 % of a step of 16 meshes)
+  float crit_above;
 };
 
 // parameter k of a double/float pair in the stencil precision T
@@ -69,10 +72,10 @@ inline void fill_float_params(DevModel& m) {
 // interval of two of its values; a kernel looks whether its values reach beyond one (a state
 // written in place, or one that the safeguard has reported) and then takes the loop. 2D only:
 // a 1D end value may lie outside. Blended Buckley-Leverett step at 4096^2: 3.94 ms without
-// that look, 3.83 with one per row of a warp, 4.23 with one per interval, 4.19 with three
+// that look, 3.87 with one per row of a warp, 4.23 with one per interval, 4.19 with three
 // slots, enough for all extrema on the line.
 inline void fill_few_criticals(DevModel& m, bool limiter, int dim) {
-  m.crit_few = limiter && dim == 2 ? 1 : 0;
+  bool few = limiter && dim == 2;
   m.crit_below = -INFINITY;
   m.crit_above = INFINITY;
   const double margin = 1e-5 * (fabs(m.umin) > fabs(m.umax) ? fabs(m.umin) : fabs(m.umax));
@@ -92,12 +95,16 @@ inline void fill_few_criticals(DevModel& m, bool limiter, int dim) {
         continue;
       }
       if (n == 2) {
-        m.crit_few = 0;
+        few = false;
         break;
       }
       m.critf2[d][n] = m.critf[d][k];
       m.critvf2[d][n++] = m.critvf[d][k];
     }
+  }
+  if (!few) {
+    m.crit_below = INFINITY;
+    m.crit_above = -INFINITY;
   }
 }
 

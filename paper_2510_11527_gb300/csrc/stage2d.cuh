@@ -433,7 +433,7 @@ __device__ __forceinline__ void stage_tile(const DevModel& m, const StageArgs2D<
       for_segs<NT>(p1_qu, p1_pts, p1_ctr);
     }
   });
-  if constexpr (FEW) few = !__syncthreads_or(beyond) && m.crit_few;
+  if constexpr (FEW) few = !__syncthreads_or(beyond);
   else __syncthreads();
 
   // ---- P2: high-order residuals, Simpson fluxes, DC potentials, LLF fluxes -------------

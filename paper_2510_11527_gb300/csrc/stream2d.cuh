@@ -68,7 +68,6 @@ struct RowSlot {
   // theta^{d,s}_1 of the cell, low-order residuals of the row's x-lines (V, X, Y)
   T s2, tc1, td1, LV1, LX1, LY1;
   T FVX;   // LLF flux (y) between V of the row below and X of this row
-  bool in;  // FP32 Buckley-Leverett: no value of the warp's row reaches beyond the slots' extrema
 };
 
 // f_l, |f_l'| and a at one value: returns f_1 in f1, f_2 in f2, |f_1'| in d1, |f_2'| in d2
@@ -181,10 +180,14 @@ __device__ __forceinline__ RowIn<T> load_row(const StageArgs2D<T>& A, size_t g) 
 }
 
 // One step: input row r arrives (in), slots p2 (row r-2), p1 (row r-1), cur (row r;
-// held row r-3 before). Finalises the cells of row r-2 if they belong to the strip.
+// held row r-3 before). Finalises the cells of row r-2 if they belong to the strip. FP32
+// Buckley-Leverett: within says whether no value of the warp's row r-1 reaches beyond the
+// slots' extrema (see fill_few_criticals), and leaves with row r's answer; it is no member of
+// the row slots, where it cost the other fluxes 3 to 8 %.
 template <int FLUX, int DIFF, class T, int BK>
 __device__ __forceinline__ void stream_step(const StreamCtx<FLUX, DIFF, T>& c, int r, const RowIn<T>& in,
-                                            const OutIn<T>& oin, RowSlot<T>& p2, RowSlot<T>& p1, RowSlot<T>& cur) {
+                                            const OutIn<T>& oin, RowSlot<T>& p2, RowSlot<T>& p1, RowSlot<T>& cur,
+                                            bool& within) {
   const DevModel& m = c.m;
   const StageArgs2D<T>& A = c.A;
   const StreamScal<T>& k = c.k;
@@ -201,9 +204,10 @@ __device__ __forceinline__ void stream_step(const StreamCtx<FLUX, DIFF, T>& c, i
   // slots' extrema (uniform over the warp)
   bool few = false;
   if constexpr (BL && sizeof(T) == 4) {
-    cur.in = __all_sync(0xffffffffu, (fmn(min3(cur.V, cur.X, cur.Y), cur.U) >= m.crit_below) &
-                                         (fmx(max3(cur.V, cur.X, cur.Y), cur.U) <= m.crit_above));
-    few = m.crit_few && cur.in && p1.in;
+    const bool here = __all_sync(0xffffffffu, (fmn(min3(cur.V, cur.X, cur.Y), cur.U) >= m.crit_below) &
+                                                  (fmx(max3(cur.V, cur.X, cur.Y), cur.U) <= m.crit_above));
+    few = here && within;
+    within = here;
   }
   const T Xm = shup(cur.X);
   cur.Vm = shup(cur.V);
@@ -561,6 +565,7 @@ __device__ __forceinline__ void stream_run(const DevModel& m, const StageArgs2D<
     return o;
   };
   OutIn<T> oin = out_in(r0);
+  bool within = false;
   if constexpr (BK != 0) {
     // the blended step is too large to unroll three times (the unrolled loop misses the
     // instruction cache): one step per iteration, the slots rotated by copies
@@ -568,7 +573,7 @@ __device__ __forceinline__ void stream_run(const DevModel& m, const StageArgs2D<
     for (int r = r0; r <= r1; ++r) {
       const RowIn<T> nin = next_row();
       const OutIn<T> noin = out_in(r + 1);
-      stream_step<FLUX, DIFF, T, BK>(c, r, in, oin, s1, s2, s0);
+      stream_step<FLUX, DIFF, T, BK>(c, r, in, oin, s1, s2, s0, within);
       const RowSlot<T> t = s1;
       s1 = s2;
       s2 = s0;
@@ -581,7 +586,7 @@ __device__ __forceinline__ void stream_run(const DevModel& m, const StageArgs2D<
       {
         const RowIn<T> nin = next_row();
         const OutIn<T> noin = out_in(r + 1);
-        stream_step<FLUX, DIFF, T, BK>(c, r, in, oin, s1, s2, s0);
+        stream_step<FLUX, DIFF, T, BK>(c, r, in, oin, s1, s2, s0, within);
         in = nin;
         oin = noin;
       }
@@ -589,7 +594,7 @@ __device__ __forceinline__ void stream_run(const DevModel& m, const StageArgs2D<
       {
         const RowIn<T> nin = next_row();
         const OutIn<T> noin = out_in(r + 2);
-        stream_step<FLUX, DIFF, T, BK>(c, r + 1, in, oin, s2, s0, s1);
+        stream_step<FLUX, DIFF, T, BK>(c, r + 1, in, oin, s2, s0, s1, within);
         in = nin;
         oin = noin;
       }
@@ -597,7 +602,7 @@ __device__ __forceinline__ void stream_run(const DevModel& m, const StageArgs2D<
       {
         const RowIn<T> nin = next_row();
         const OutIn<T> noin = out_in(r + 3);
-        stream_step<FLUX, DIFF, T, BK>(c, r + 2, in, oin, s0, s1, s2);
+        stream_step<FLUX, DIFF, T, BK>(c, r + 2, in, oin, s0, s1, s2, within);
         in = nin;
         oin = noin;
       }
