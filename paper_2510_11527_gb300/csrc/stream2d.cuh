@@ -671,8 +671,8 @@ __device__ __forceinline__ void blend_s_tile(const double* __restrict__ ub, int 
 // the strip height of a single mesh (strip_plan.h)
 static StripPlan stream_plan(int nx, int ny, bool heavy, bool zero) {
   const int bands = (nx + STREAM_BAND - 1) / STREAM_BAND;
-  return strip_plan(heavy ? MARCH_HEAVY : (zero ? MARCH_ZERO : MARCH_LIGHT),
-                    [=](int S) { return (long long)bands * ((ny + S - 1) / S); });
+  if (!heavy && !zero) return strip_plan_light(bands, ny);
+  return strip_plan(heavy ? MARCH_HEAVY : MARCH_ZERO, [=](int S) { return (long long)bands * ((ny + S - 1) / S); });
 }
 
 // the stage arguments of output o alone

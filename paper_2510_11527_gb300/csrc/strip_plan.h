@@ -8,11 +8,20 @@
 // (degenerate Burgers 2048^2, per step: 0.44 ms with 16 to 26 rows, 0.48 with 32, 0.56 with
 // 64 in one wave). The heavy kernels' strips are alike, so for them whole waves count (the
 // busiest SM's CTAs, R at a time) more than the work (blended Buckley-Leverett 2048^2: 28
-// rows, 3.0 waves, 1.14 ms; 26 rows 1.26 ms; 4096^2: 84 rows 3.94, 56 rows 4.03 ms), and
+// rows, 3.0 waves, 1.14 ms; 26 rows 1.26 ms; 4096^2: 84 rows 3.87, 56 rows 4.03 ms), and
 // for a batch's items as much (16 meshes, 5.6 million cells, one step: 29 rows 617, 23 rows
-// 642 us). Measured per stage against the fixed number of waves used before: Burgers 100^2
-// 23 -> 12 us, 512^2 25 -> 17 us; Buckley-Leverett 1024^2 101 -> 54 us (with its loop-free
-// wave speeds).
+// 642 us). Against a fixed number of waves: Burgers 100^2 23 -> 12 us per stage, 512^2 128
+// -> 85 us per step; Buckley-Leverett 1024^2 101 -> 54 us per stage (with its loop-free wave
+// speeds).
+//
+// For the light kernel on a single mesh the estimate is flat around its minimum, where what
+// counts is how the fronts fall into strips: two and a half waves of strips of 16 to 48 rows
+// are the choice unless it predicts at least 5 % less (up to about 900^2; at 850^2 it
+// predicts 7.5 %, at 1024^2 2.5 %). Degenerate Burgers, us per step on fresh discs / after
+// 300 steps, by the estimate alone and so: 1024^2 169 / 166 and 162 / 175, 1200 x 1100 193 /
+// 199 and 182 / 194, 300 x 4000 202 / 199 and 191 / 184, 2200^2 508 / 496 and 492 / 476,
+// 3000^2 851 / 836 and 827 / 810, 4096^2 1471 / 1453 and 1481 / 1461. Taller strips at two
+// and a half waves (100 rows at 4096^2) took 1491 / 1463 there.
 #pragma once
 
 namespace af {
@@ -33,19 +42,33 @@ constexpr MarchKind MARCH_HEAVY = {3, {0.68, 0.82, 1.00, 0.0}, 0.7, 0.5};    // 
 constexpr MarchKind MARCH_ITEMS = {4, {1.12, 1.25, 1.50, 1.72}, 0.5, 0.5};   // a batch's items, dealt to one wave
 constexpr MarchKind MARCH_PAIR = {3, {1.22, 1.40, 1.69, 0.0}, 0.0, 1.0};     // two columns per lane (zero flux)
 
+// estimated time of w strips of S rows
+inline double strip_cost(const MarchKind& k, int S, long long w) {
+  const long long q = (w + 4 * 152 * 97 / 100) / (4 * 152);   // CTAs of the busiest SM, but for a few
+  const int rest = (int)(q % k.R);
+  const double waves = (double)(q / k.R) * k.t[k.R - 1] + (rest ? k.t[rest - 1] : 0.0);
+  const double work = (double)w / (4 * 152) * k.t[k.R - 1] / k.R;
+  return (S + 5) * (k.waves * waves + (1.0 - k.waves) * work + k.tail * k.t[0]);
+}
+
 // warps(S): how many warps strips of S rows make
 template <class F>
 inline StripPlan strip_plan(const MarchKind& k, F&& warps) {
   StripPlan best{4, -1.0};
   for (int S = 4; S <= 128; S += S < 32 ? 1 : 4) {
-    const long long w = warps(S), q = (w + 4 * 152 * 97 / 100) / (4 * 152);   // CTAs of the busiest SM, but for a few
-    const int rest = (int)(q % k.R);
-    const double waves = (double)(q / k.R) * k.t[k.R - 1] + (rest ? k.t[rest - 1] : 0.0);
-    const double work = (double)w / (4 * 152) * k.t[k.R - 1] / k.R;
-    const double cost = (S + 5) * (k.waves * waves + (1.0 - k.waves) * work + k.tail * k.t[0]);
+    const double cost = strip_cost(k, S, warps(S));
     if (best.cost < 0.0 || cost < best.cost) best = StripPlan{S, cost};
   }
   return best;
+}
+
+// the light kernel on a single mesh of `bands` bands and ny rows
+inline StripPlan strip_plan_light(long long bands, int ny) {
+  const StripPlan p = strip_plan(MARCH_LIGHT, [=](int S) { return bands * ((ny + S - 1) / S); });
+  const long long slots = 152 * 16 * 5 / 2, rows = (bands * ny + slots - 1) / slots;
+  const int S = rows < 16 ? 16 : (rows > 48 ? 48 : (int)rows);
+  const double cost = strip_cost(MARCH_LIGHT, S, bands * ((ny + S - 1) / S));
+  return p.cost < 0.95 * cost ? p : StripPlan{S, cost};
 }
 
 }  // namespace af
