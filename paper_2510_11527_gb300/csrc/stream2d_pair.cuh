@@ -16,7 +16,8 @@
 // A packed operation rounds each half as the scalar one does. Where the scalar code
 // negates an operand the packed one uses the mirrored form -(a b - c) = (-a) b + c with
 // coefficients negated once (rounding to nearest is symmetric), so results differ at most
-// in the sign of a zero. The convection terms, exact zeros, are not formed.
+// in the sign of a zero. The convection terms, exact zeros, are not formed (of an unlimited
+// state that has overflowed FP32 they make some infinities NaN).
 #pragma once
 #include "stream2d.cuh"
 

@@ -76,3 +76,56 @@ def test_mass_is_conserved_exactly(ny, flux, diff):
         s.forward_euler(0.5 * s.dt_cfl())
         got = s.get_state()[0]
     assert abs(math.fsum(got.ravel()) - math.fsum(st[0].ravel())) <= got.size * 2.0 ** -52
+
+
+def _device_arrays(b, spec):
+    """The device arrays (FP64 averages, FP32 points) of a batch's first mesh."""
+    import torch
+    from paper_2510_11527_gb300 import capi
+
+    def view(ptr, kind):
+        class _View:
+            __cuda_array_interface__ = {"shape": (spec.ny, spec.nx), "typestr": kind, "data": (ptr, False), "version": 3}
+        return torch.as_tensor(_View(), device="cuda")
+
+    ptrs, _ = capi.af_batch_device_ptrs(b, 0)
+    return [view(p, "<f8" if k == 0 else "<f4") for k, p in enumerate(ptrs)]
+
+
+@pytest.mark.parametrize("nx", [1259, 1260, 1261])
+@pytest.mark.parametrize("diff", ["const", "pme2", "pme3", "pwl", "cubic", "ramp"])
+@pytest.mark.parametrize("rk,limiter", [(3, True), (54, True), (3, False)])
+def test_two_columns_equal_one_column(nx, diff, rk, limiter):
+    """The mesh's size decides between one and two columns per lane, so both have to give the
+    same bits (a zero's sign aside). A batch marches with one column per lane at every size:
+    two steps of a batch of one mesh against the single mesh."""
+    from paper_2510_11527_gb300 import capi
+    spec = mesh(nx, 1200, "zero", diff, limiter)
+    st = [a.numpy() for a in ai.random_state_2d(spec, seed=nx + rk)]
+    f, d = capi.af_flux(), capi.af_diff()
+    f.kind, d.kind = capi.FLUX["zero"], capi.DIFF[spec.diff[0]]
+    for k, v in enumerate(spec.diff[1]):
+        d.p[k] = v
+    b = capi.af_batch_create([capi.af_grid(2, spec.nx, spec.ny, spec.x0, spec.x1, spec.y0, spec.y1)], [f], [d],
+                             [capi.af_bounds_t(spec.umin, spec.umax, 0)],
+                             capi.af_opts(capi.PREC["fp32_mixed"], rk, 0.0, 0.0, int(limiter), 0, 1.0))
+    try:
+        capi.af_batch_set_state(b, 0, spec.cells, *st)
+        capi.af_batch_step(b, 2)
+        capi.af_batch_sync(b)
+        want, t = [a.cpu().numpy() for a in _device_arrays(b, spec)], capi.af_batch_time(b, 0)
+    finally:
+        capi.af_batch_destroy(b)
+    with solver(spec, rk) as s:
+        s.set_state(st)
+        for _ in range(2):
+            s.step(0.0)
+        assert s.time() == t > 0.0
+        got = [a.cpu().numpy() for a in s.device_tensors()]
+    assert float(np.max(np.abs(got[0] - st[0]))) > 1e-3
+    # the arrays as they are on the device. An unlimited run of the cubic potential, which is
+    # unstable outside [0, 1], overflows FP32; there one column forms the convection terms,
+    # zero times an infinity, and holds a NaN where two columns hold the infinity
+    for g, w in zip(got, want):
+        finite = np.isfinite(w)
+        assert np.array_equal(finite, np.isfinite(g)) and np.array_equal(g[finite], w[finite])
