@@ -13,10 +13,10 @@
 // points of layer r - 1, the z-limiter works on cell r - 1 and the averages of layer r - 2
 // are finished.
 //
-// FP64 form: a cell's 27 half-spaced locations enter its centre and its three potentials
-// only through 8 sums (the centre; the pairs of x-, y- and z-faces; the fours of xy-, xz-
-// and yz-edges; the 8 corners), each built from sums along one axis after another: 19
-// additions and 8 operations per direction instead of 27 weighted terms per direction.
+// FP64 form (zero flux): a cell's 27 half-spaced locations enter its centre and its three
+// potentials only through 8 sums (the centre; the pairs of x-, y- and z-faces; the fours of
+// xy-, xz- and yz-edges; the 8 corners), each built from sums along one axis after another:
+// 19 additions and 8 operations per direction instead of 27 weighted terms per direction.
 //
 // FP32-mixed form: stencils and limiters in FP32; the averages are updated from the widened
 // face values in FP64 (differences, products with mu and nu, sums). That costs: with the
@@ -132,14 +132,14 @@ struct Incr {
 
 // What a layer leaves for the one above it: sums over its upper plane of z-faces. The FP64
 // form adds the 27 locations by kind (see the top of this file): the z-face, the pairs of
-// xz- and yz-edges and the four corners of z and a, and the flux sums. The FP32 form keeps
+// xz- and yz-edges and the four corners of z and a. The FP32 form keeps
 // the order of the weighted 27-term sums, whose rounding shows in FP32: their first nine
 // (three) terms, and the plane's nine values of a.
 template <class T> struct M3Level;
 template <> struct M3Level<double> {
-  double z[4], a[4], f[4];
+  double z[4], a[4];
   __device__ __forceinline__ void clear() {
-    for (int k = 0; k < 4; ++k) z[k] = a[k] = f[k] = 0.0;
+    for (int k = 0; k < 4; ++k) z[k] = a[k] = 0.0;
   }
 };
 template <> struct M3Level<float> {
@@ -246,7 +246,6 @@ __device__ __forceinline__ void m3_limit(const DevModel& m, const M3Scal<T>& k, 
   bool out;
   if constexpr (sizeof(T) == 8) {
     out = !(inb(h0, k.umin, k.umax) & inb(h1, k.umin, k.umax) & inb(h2, k.umin, k.umax) & inb(h3, k.umin, k.umax));
-    if constexpr (FLUX != FLUX_ZERO) out |= !(inb(gp, k.umin, k.umax) & inb(gm, k.umin, k.umax));
   } else {
     T lo = fmn(fmn(h0, h1), fmn(h2, h3)), hi = fmx(fmx(h0, h1), fmx(h2, h3));
     if constexpr (FLUX != FLUX_ZERO) {
@@ -288,6 +287,7 @@ __global__ void __launch_bounds__(32 * TY, 1)
     march3d_kernel(const DevModel m, const __grid_constant__ StageArgs3D<T> A, int o, int S, int bands, int rows) {
   using SH = M3Shared<FLUX, T, TY>;
   constexpr bool CONV = FLUX != FLUX_ZERO;
+  static_assert(sizeof(T) == 4 || !CONV, "FP64 meshes with a flux take the four kernels (march3d_takes)");
   extern __shared__ __align__(16) unsigned char m3_raw[];
   SH& sh = *reinterpret_cast<SH*>(m3_raw);
   const double dtv = *A.dt;
@@ -532,22 +532,6 @@ __global__ void __launch_bounds__(32 * TY, 1)
           AHx = sfma(T(8), sfma(T(16), a[0], sfma(T(4), b2 + Fz, Eyz)), -sfma(T(16), b1, sfma(T(4), b3 + Exz, V))) * r216;
           AHy = sfma(T(8), sfma(T(16), a[0], sfma(T(4), b1 + Fz, Exz)), -sfma(T(16), b2, sfma(T(4), b3 + Eyz, V))) * r216;
           AHz = sfma(T(8), sfma(T(16), a[0], sfma(T(4), b1 + b2, b3)), -sfma(T(16), Fz, sfma(T(4), Exz + Eyz, V))) * r216;
-        }
-        if constexpr (CONV) {
-          // Simpson averages of f_l over the upper faces
-          auto f = [&](int l, T v) { return flux<FLUX, T>(m, l, v); };
-          const T r36 = T(1.0 / 36.0);
-          const T y37 = f(0, zm7) + f(0, z[7]);
-          FHx = sfma(T(16), f(0, z[1]), sfma(T(4), (f(0, zm3) + f(0, z[3])) + (lv.f[0] + f(0, z[5])), lv.f[1] + y37)) * r36;
-          lv.f[0] = f(0, z[5]);
-          lv.f[1] = y37;
-          const T f3 = f(1, z[3]), f7 = f(1, z[7]);
-          const T x7 = shup(f7) + f7;
-          FHy = sfma(T(16), f(1, z[2]), sfma(T(4), (shup(f3) + f3) + (lv.f[2] + f(1, z[6])), lv.f[3] + x7)) * r36;
-          lv.f[2] = f(1, z[6]);
-          lv.f[3] = x7;
-          const T h5 = f(2, z[5]), h7 = f(2, zm7) + f(2, z[7]);
-          FHz = sfma(T(16), f(2, z[4]), sfma(T(4), (shup(h5) + h5) + (f(2, zm6) + f(2, z[6])), shup(h7) + h7)) * r36;
         }
       }
       if (xy) {

@@ -9,8 +9,8 @@ constexpr int M3_BAND = 28;   // output columns per tile
 
 // Rows per CTA, the larger and the smaller choice. The CTA's registers are the SM's: 16
 // rows at 128, 12 at 168 and 8 at 255 registers per thread; more rows cost fewer halo rows
-// per output row, fewer registers spill (porous medium 80^3 FP64 at 8 / 12 rows: 2.85 / 2.67 ms per SSP-RK(5,4) step). The
-// smaller one is for meshes that leave SMs without a tile.
+// per output row, fewer registers spill (porous medium 80^3 FP64 at 8 / 12 rows: 2.85 / 2.67
+// ms per SSP-RK(5,4) step). The smaller one is for meshes that leave SMs without a tile.
 constexpr int m3_rows(int flux, bool fp64) { return fp64 ? 12 : (flux == AF_FLUX_ZERO ? 16 : 12); }
 constexpr int M3_ROWS_SMALL = 8;
 
@@ -45,14 +45,14 @@ inline M3Plan m3_plan(const int* n, int TY) {
 }
 
 // Whether a mesh's stage without the blend marches. FP32-mixed always does (128^3 zero /
-// Burgers flux: 1922 -> 507 / 2101 -> 732 us per step; 20^3: 165 -> 42 us). FP64 is bound
+// Burgers flux: 1922 -> 534 / 2101 -> 824 us per step; 20^3: 165 -> 42 us). FP64 is bound
 // by the FP64 unit, and a marching tile repeats work in its halo: with a flux (six LLF
-// fluxes per cell instead of three, 8 rows per CTA for lack of registers) the four kernels
-// are faster from 40^3 on (128^3: 13.2 against 15.9 ms per step); without one (porous
-// medium) it depends on how well the mesh fills tiles of 28 columns: a stage takes about
-// 55 us + 1.13 ns per cell in four kernels and 4 us + m3_plan's cost here (33^3: 97 / 106
-// us; 40 x 45 x 26: 104 / 100; 21 x 102 x 61: 215 / 178; 128^3: 2377 / 2161; 20^3: 80 / 42);
-// it marches where that predicts at least 3 % less.
+// fluxes per cell instead of three, only 8 rows per CTA for lack of registers) the four
+// kernels were faster from 40^3 on (128^3: 13.2 against 15.9 ms per step), and the march has
+// no such form; without one (porous medium) it depends on how well the mesh fills tiles of 28
+// columns: a stage takes about 55 us + 1.13 ns per cell in four kernels and 4 us + m3_plan's
+// cost here (33^3: 97 / 106 us; 40 x 45 x 26: 104 / 100; 21 x 102 x 61: 215 / 178; 128^3:
+// 2377 / 2161; 20^3: 80 / 42); it marches where that predicts at least 3 % less.
 inline bool march3d_takes(int flux, bool fp64, const int* n) {
   if (!fp64) return true;
   if (flux != AF_FLUX_ZERO) return false;
