@@ -170,7 +170,7 @@ af_status af_device_ptrs_arrays(af_ctx* ctx, int narr, void** ptrs, int dtype[2]
  * rectangle with ends: its padded device layout, (nx+1) x (ny+1) entries per array,
  * entry (I, J) holding the average of cell (I-1, J-1) and the corner / edge values at
  * that cell's top-right; the averages in row and column 0, X in row 0 and Y in column 0
- * are not DoFs). */
+ * are not DoFs). What is written through them is not checked as af_set_state checks. */
 af_status af_device_ptrs(af_ctx* ctx, void* ptrs[4], int dtype[2]);
 
 /* Per-cell external smoothness indicator s (nx*ny doubles, host) used when

@@ -443,7 +443,7 @@ __device__ __forceinline__ bool inb(T z, T umin, T umax) {
 // min of Theta over two / four (zL, zH) pairs. The common case (every zH inside the
 // bounds, so the minimum is 1) is tested first: in FP64 with integer compares, in FP32 by
 // the least and the largest zH (rectangle of Example 6.9, one FP32 step at 1536^2: 495 ->
-// 477 us; a NaN among them counts as inside in both forms).
+// 477 us).
 template <class T>
 __device__ __forceinline__ T theta_pair(T a0, T a1, T b0, T b1, T umin, T umax) {
   if constexpr (sizeof(T) == 8)
