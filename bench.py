@@ -56,10 +56,10 @@ FLOPS_PER_CELL_STAGE_3D = 791.56
 # the ncu captures summarised in profiles/stage2d_fp64_degenerate_burgers_1024.md and
 # profiles/stream2d_fp32mixed_degenerate_burgers_2048.md, keyed by (precision, n); null
 # for any other size.
-NCU_TRAFFIC_PER_LAUNCH = {("fp64", 1024): 74.79e6, ("fp32_mixed", 2048): 229.67e6}
+NCU_TRAFFIC_PER_LAUNCH = {("fp64", 1024): 74.74e6, ("fp32_mixed", 2048): 229.73e6}
 # thread instructions per cell-stage of the FP32-mixed (column-marching) stage from the
 # same capture (smsp__inst_executed.sum x 32 / cells)
-NCU_INSTR_PER_CELL_STAGE = {("fp32_mixed", 2048): 769.0}
+NCU_INSTR_PER_CELL_STAGE = {("fp32_mixed", 2048): 764.0}
 
 
 def load_peaks():
