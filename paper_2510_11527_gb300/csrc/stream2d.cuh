@@ -671,7 +671,7 @@ __device__ __forceinline__ void blend_s_tile(const double* __restrict__ ub, int 
 // the strip height of a single mesh (strip_plan.h)
 static StripPlan stream_plan(int nx, int ny, bool heavy, bool zero) {
   const int bands = (nx + STREAM_BAND - 1) / STREAM_BAND;
-  if (!heavy && !zero) return strip_plan_light(bands, ny);
+  if (!heavy && !zero) return StripPlan{strip_rows_light(bands, ny), 0.0};
   return strip_plan(heavy ? MARCH_HEAVY : MARCH_ZERO, [=](int S) { return (long long)bands * ((ny + S - 1) / S); });
 }
 

@@ -14,14 +14,8 @@
 // -> 85 us per step; Buckley-Leverett 1024^2 101 -> 54 us per stage (with its loop-free wave
 // speeds).
 //
-// For the light kernel on a single mesh the estimate is flat around its minimum, where what
-// counts is how the fronts fall into strips: two and a half waves of strips of 16 to 48 rows
-// are the choice unless it predicts at least 5 % less (up to about 900^2; at 850^2 it
-// predicts 7.5 %, at 1024^2 2.5 %). Degenerate Burgers, us per step on fresh discs / after
-// 300 steps, by the estimate alone and so: 1024^2 169 / 166 and 162 / 175, 1200 x 1100 193 /
-// 199 and 182 / 194, 300 x 4000 202 / 199 and 191 / 184, 2200^2 508 / 496 and 492 / 476,
-// 3000^2 851 / 836 and 827 / 810, 4096^2 1471 / 1453 and 1481 / 1461. Taller strips at two
-// and a half waves (100 rows at 4096^2) took 1491 / 1463 there.
+// The light kernel on a single mesh (Burgers, linear flux) is the exception: the estimate is
+// flat around its minimum there, and what counts is how the last wave ends (strip_rows_light).
 #pragma once
 
 namespace af {
@@ -36,8 +30,7 @@ struct MarchKind {
   double t[4];
   double waves, tail;   // weights of the waves (against the work) and of the tail
 };
-constexpr MarchKind MARCH_LIGHT = {4, {1.12, 1.25, 1.50, 1.72}, 0.0, 1.0};   // one column per lane
-constexpr MarchKind MARCH_ZERO = {4, {1.05, 1.18, 1.40, 1.60}, 0.0, 1.0};    // the same, zero flux
+constexpr MarchKind MARCH_ZERO = {4, {1.05, 1.18, 1.40, 1.60}, 0.0, 1.0};    // one column per lane, zero flux
 constexpr MarchKind MARCH_HEAVY = {3, {0.68, 0.82, 1.00, 0.0}, 0.7, 0.5};    // Buckley-Leverett, blends (relative)
 constexpr MarchKind MARCH_ITEMS = {4, {1.12, 1.25, 1.50, 1.72}, 0.5, 0.5};   // a batch's items, dealt to one wave
 constexpr MarchKind MARCH_PAIR = {3, {1.22, 1.40, 1.69, 0.0}, 0.0, 1.0};     // two columns per lane (zero flux)
@@ -62,13 +55,22 @@ inline StripPlan strip_plan(const MarchKind& k, F&& warps) {
   return best;
 }
 
-// the light kernel on a single mesh of `bands` bands and ny rows
-inline StripPlan strip_plan_light(long long bands, int ny) {
-  const StripPlan p = strip_plan(MARCH_LIGHT, [=](int S) { return bands * ((ny + S - 1) / S); });
-  const long long slots = 152 * 16 * 5 / 2, rows = (bands * ny + slots - 1) / slots;
-  const int S = rows < 16 ? 16 : (rows > 48 ? 48 : (int)rows);
-  const double cost = strip_cost(MARCH_LIGHT, S, bands * ((ny + S - 1) / S));
-  return p.cost < 0.95 * cost ? p : StripPlan{S, cost};
+// Strip height of the light kernel on a single mesh of `bands` bands and ny rows: one and a
+// quarter waves of 16 warps per SM as long as 4 to 16 rows give them, else two and a half of
+// at most 48 rows. Both leave the SMs that are done early a short rest; full last waves, and
+// those that end at a half between, wait for the strips along fronts. Degenerate Burgers, us
+// per step on fresh discs / after 300 steps, as the estimate would choose and so: 512^2 85 /
+// 92 and 79 / 88, 950^2 159 / 151 and 143 / 154, 1024^2 169 / 166 and 159 / 170, 1250^2 218 /
+// 223 and 211 / 208, 300 x 4000 201 / 198 and 193 / 186, 2048^2 439 / 427 both, 3000^2 851 /
+// 836 and 827 / 810, 4096^2 1471 / 1453 and 1481 / 1461 (with 100 rows, two and a half waves
+// there, 1491 / 1463). Over 26 meshes from 200^2 to 4096^2 within 0.4 % of two and a half
+// waves of 16 to 128 rows, the rule before, or faster, and within 3 % of the estimate.
+inline int strip_rows_light(long long bands, int ny) {
+  constexpr long long wave = 152 * 16;
+  auto rows = [=](long long warps) { return (bands * ny + warps - 1) / warps; };
+  const long long one = rows(wave * 5 / 4), two = rows(wave * 5 / 2);
+  if (one <= 16) return one < 4 ? 4 : (int)one;
+  return two > 48 ? 48 : (int)two;
 }
 
 }  // namespace af

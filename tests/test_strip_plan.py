@@ -1,6 +1,6 @@
 """Strip heights of the light column-marching kernel (host code, compiled with the host
-compiler): the estimate's choice where it predicts at least 5 % less than two and a half
-waves of 16 to 48 rows, else these."""
+compiler): one and a quarter waves of warps as long as 4 to 16 rows give them, else two and
+a half of at most 48 rows."""
 import os
 import subprocess
 
@@ -14,16 +14,13 @@ int main() {
   for (int nx : {28, 100, 300, 512, 850, 1024, 1300, 2048, 3000, 4096, 20000})
     for (int ny : {1, 4, 100, 300, 512, 850, 1024, 1300, 2048, 3000, 4096, 20000}) {
       const long long bands = (nx + 27) / 28;
-      const auto warps = [&](int S) { return bands * ((ny + S - 1) / S); };
-      const af::StripPlan p = af::strip_plan_light(bands, ny), best = af::strip_plan(af::MARCH_LIGHT, warps);
-      const double cost = af::strip_cost(af::MARCH_LIGHT, p.S, warps(p.S));
-      bool ok = p.S >= 4 && p.S <= 128 && p.cost == cost && best.cost >= 0.95 * p.cost - 1e-9;
-      if (p.S != best.S) {   // two and a half waves of 16 warps per SM, as far as 16 to 48 rows give them
-        const double waves = (double)bands * ny / p.S / (152 * 16);
-        ok = ok && p.S >= 16 && p.S <= 48 && (p.S == 48 || waves <= 2.5) && (p.S == 16 || waves >= 2.3);
-      }
+      const int S = af::strip_rows_light(bands, ny);
+      const double waves = (double)bands * ny / S / (152 * 16), shorter = (double)bands * ny / (S - 1) / (152 * 16);
+      const double want = (double)bands * ny / 16 / (152 * 16) <= 1.25 ? 1.25 : 2.5;
+      // the shortest strips that make no more waves than wanted
+      bool ok = S >= 4 && S <= 48 && (waves <= want || S == 48) && (shorter > want || S == 4);
       if (!ok) {
-        std::printf("%d x %d: %d rows (estimate's choice %d)\n", nx, ny, p.S, best.S);
+        std::printf("%d x %d: %d rows, %.2f waves\n", nx, ny, S, waves);
         return 1;
       }
     }
